@@ -3,13 +3,14 @@
 // point, k = 4 in the paper), exact, on a hashed uniform grid.
 //
 //   1. bounding box (float min/max as ordered integers, atomics)
-//   2. cell size h: the median k-NN distance of 256 sampled points, each found
-//      by one block scanning the whole cloud (the only host synchronisation)
-//   3. counting sort of the points by the hash of their cell
-//   4. per point: visit cells in shells of growing Chebyshev radius r around
-//      its own, keep the k smallest squared distances, and stop once the k-th
-//      is <= (r h)^2 (no point outside the visited cube can be closer); the
-//      work per point is bounded (see k_query).
+//   2. cell size h: 1.5 times the median k-NN distance of 256 sampled points,
+//      exact (k_sample_bound, k_sample_scan, k_sample_select; the only host
+//      synchronisation follows)
+//   3. counting sort of the points by the hash of their search cell (1.6 h)
+//   4. per point, in sorted order: the 8 search cells nearest to it (k_query);
+//      points that these do not settle search a wider cube (k_query_far)
+// 5M points on 50 surfaces: 8.73 ms with one block per sample and the points
+// queried in input order cell by cell, 1.14 ms now.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -35,7 +36,7 @@ __device__ __forceinline__ float unordered(uint32_t o) {
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-__global__ void k_bbox(const float* __restrict__ xyz, int64_t n, uint32_t* box) {
+__global__ void __launch_bounds__(256) k_bbox(const float* __restrict__ xyz, int64_t n, uint32_t* box) {
   uint32_t lo[3] = {0xffffffffu, 0xffffffffu, 0xffffffffu}, hi[3] = {0u, 0u, 0u};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     for (int d = 0; d < 3; ++d) {
@@ -43,17 +44,33 @@ __global__ void k_bbox(const float* __restrict__ xyz, int64_t n, uint32_t* box) 
       lo[d] = min(lo[d], o);
       hi[d] = max(hi[d], o);
     }
+  // one atomic per block and bound: 58 thousand same-address atomics of a
+  // warp each took 51 us on 5M points, whose 60 MB are a 9 us read
+  __shared__ uint32_t s_lo[3][8], s_hi[3][8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int d = 0; d < 3; ++d) {
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-      lo[d] = min(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], s));
-      hi[d] = max(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], s));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      atomicMin(box + d, lo[d]);
-      atomicMax(box + 3 + d, hi[d]);
+    const uint32_t l = __reduce_min_sync(0xffffffffu, lo[d]), h = __reduce_max_sync(0xffffffffu, hi[d]);
+    if (lane == 0) {
+      s_lo[d][warp] = l;
+      s_hi[d][warp] = h;
     }
   }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    uint32_t l = 0xffffffffu, h = 0u;
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+      l = min(l, s_lo[threadIdx.x][w]);
+      h = max(h, s_hi[threadIdx.x][w]);
+    }
+    atomicMin(box + threadIdx.x, l);
+    atomicMax(box + 3 + threadIdx.x, h);
+  }
+}
+
+// The squared distance, one fixed sequence of operations: the sample kernels
+// compare values that different kernels computed.
+__device__ __forceinline__ float dist2(float dx, float dy, float dz) {
+  return fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
 }
 
 // keep the k smallest values of a sorted ascending list
@@ -67,56 +84,266 @@ __device__ __forceinline__ void insert_k(float* best, int k, int& m, float d2) {
   best[q] = d2;
 }
 
-// One block per sampled point: the k smallest squared distances over the cloud.
-__global__ void __launch_bounds__(256) k_sample_knn(const float* __restrict__ xyz, int64_t n, int k, float* out) {
-  __shared__ float s_best[256 * kMaxK];
-  const int64_t si = (int64_t)blockIdx.x * n / kSamples;
+// The k-th smallest of a block's sorted lists (m entries in each thread), in
+// thread 0; INFINITY if there are fewer.  k rounds of taking the least head,
+// first in every warp, then over the warps' lists.
+__device__ float block_kth(const float* best, int k, int m) {
+  __shared__ float s_top[32][kMaxK];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  int at = 0;
+  for (int r = 0; r < k; ++r) {  // (distances are >= 0: their bits order as they do)
+    const uint32_t head = at < m ? __float_as_uint(best[at]) : 0x7f800000u;
+    const uint32_t least = __reduce_min_sync(0xffffffffu, head);
+    const unsigned who = __ballot_sync(0xffffffffu, head == least && at < m);
+    if (who && lane == __ffs(who) - 1) ++at;
+    if (lane == 0) s_top[warp][r] = __uint_as_float(least);
+  }
+  __syncthreads();
+  float kth = INFINITY;
+  if (warp == 0) {
+    at = 0;
+    for (int r = 0; r < k; ++r) {
+      const bool more = lane < warps && at < k;
+      const uint32_t head = more ? __float_as_uint(s_top[lane][at]) : 0x7f800000u;
+      const uint32_t least = __reduce_min_sync(0xffffffffu, head);
+      const unsigned who = __ballot_sync(0xffffffffu, head == least && more);
+      if (who && lane == __ffs(who) - 1) ++at;
+      kth = __uint_as_float(least);
+    }
+  }
+  return kth;
+}
+
+__device__ __forceinline__ int64_t sample_index(int b, int64_t n) { return (int64_t)b * n / kSamples; }
+
+// The k-NN distance of the samples without 256 scans of the cloud (one block
+// per sample took 6.2 of 8.7 ms on 5M points: 1.3 G distances on 256 blocks,
+// each thread with a list in local memory):
+//   k_sample_bound   a bound per sample: the k-th smallest squared distance
+//                    to a subset -- the 8 groups of 32 consecutive points
+//                    around it and 1 / 128 of the cloud (at least 32768
+//                    points) in evenly spread groups of 32; four groups a
+//                    warp in flight (one at a time: 207 us on 5M points)
+//   k_sample_scan    every point against every sample's bound; about 128 k
+//                    points of a cloud in random order pass and are listed.
+//                    1024 points of a block first test their bounding box
+//                    against each bound: where neighbours in memory are
+//                    neighbours in space nearly every (block, sample) is
+//                    skipped, and a random order costs 7 instructions a pair.
+//   k_sample_select  the k-th smallest of the list, or of the whole cloud
+//                    where a list ran over
+// The result is the exact k-th smallest squared distance in every case.
+constexpr int kSubGroup = 32;
+constexpr int kSubLeast = 32768;   // points
+constexpr int kListCap = 4096;
+constexpr int kBoundThreads = 512;
+
+__global__ void __launch_bounds__(kBoundThreads) k_sample_bound(const float* __restrict__ xyz, int64_t n, int k, int64_t groups,
+                                                      float* bound, uint32_t* list_count) {
+  const int64_t si = sample_index(blockIdx.x, n);
   const float px = __ldg(xyz + 3 * si), py = __ldg(xyz + 3 * si + 1), pz = __ldg(xyz + 3 * si + 2);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t total = (n + kSubGroup - 1) / kSubGroup;   // groups of the cloud
+  const int64_t near0 = max((int64_t)0, min(si / kSubGroup - 4, total - 8)), near1 = min(near0 + 8, total);
   float best[kMaxK];
   int m = 0;
-  for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-    if (j == si) continue;
-    const float dx = __ldg(xyz + 3 * j) - px, dy = __ldg(xyz + 3 * j + 1) - py, dz = __ldg(xyz + 3 * j + 2) - pz;
-    insert_k(best, k, m, dx * dx + dy * dy + dz * dz);
+  // groups <= total evenly spread ones, and [near0, near1); none twice
+  constexpr int kWarps = kBoundThreads / 32;
+  const int64_t near = near1 - near0;
+  for (int64_t g0 = warp; g0 < groups + near; g0 += 4 * kWarps) {
+    float d2[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t g = g0 + u * kWarps;
+      const int64_t at = g < near ? near0 + g : (g - near) * total / groups;
+      const int64_t j = at * kSubGroup + lane;
+      const bool skip = g >= groups + near || (g >= near && at >= near0 && at < near1) || j >= n || j == si;
+      d2[u] = skip ? INFINITY
+                   : dist2(__ldg(xyz + 3 * j) - px, __ldg(xyz + 3 * j + 1) - py, __ldg(xyz + 3 * j + 2) - pz);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (d2[u] < INFINITY) insert_k(best, k, m, d2[u]);
   }
-  for (int q = 0; q < k; ++q) s_best[threadIdx.x * kMaxK + q] = q < m ? best[q] : INFINITY;
-  __syncthreads();
+  __syncwarp();
+  const float kth = block_kth(best, k, m);
   if (threadIdx.x == 0) {
-    float all[kMaxK];
-    int mm = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t)
-      for (int q = 0; q < k; ++q) {
-        const float v = s_best[t * kMaxK + q];
-        if (v == INFINITY) break;
-        insert_k(all, k, mm, v);
-      }
-    out[blockIdx.x] = mm < k ? INFINITY : sqrtf(all[k - 1]);
+    bound[blockIdx.x] = kth;
+    list_count[blockIdx.x] = 0u;
   }
 }
 
+__global__ void __launch_bounds__(256) k_sample_scan(const float* __restrict__ xyz, int64_t n,
+                                                     const float* __restrict__ bound, uint32_t* list_count,
+                                                     float* list) {
+  __shared__ float4 s_sample[kSamples];
+  __shared__ int s_pick[kSamples];
+  __shared__ float s_box[6][8];
+  __shared__ int s_n;
+  static_assert(kSamples == 256, "one thread per sample");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  {
+    const int64_t si = sample_index(threadIdx.x, n);
+    s_sample[threadIdx.x] =
+        make_float4(__ldg(xyz + 3 * si), __ldg(xyz + 3 * si + 1), __ldg(xyz + 3 * si + 2), bound[threadIdx.x]);
+  }
+  for (int64_t t0 = (int64_t)blockIdx.x * 1024; t0 < n; t0 += (int64_t)gridDim.x * 1024) {
+    float x[4], y[4], z[4];
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t j = t0 + u * 256 + threadIdx.x;
+      const bool in = j < n;
+      x[u] = in ? __ldg(xyz + 3 * j) : INFINITY;  // (an infinite distance passes no finite bound)
+      y[u] = in ? __ldg(xyz + 3 * j + 1) : INFINITY;
+      z[u] = in ? __ldg(xyz + 3 * j + 2) : INFINITY;
+      if (in) {
+        lo[0] = fminf(lo[0], x[u]); hi[0] = fmaxf(hi[0], x[u]);
+        lo[1] = fminf(lo[1], y[u]); hi[1] = fmaxf(hi[1], y[u]);
+        lo[2] = fminf(lo[2], z[u]); hi[2] = fmaxf(hi[2], z[u]);
+      }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+        hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+      }
+      if (lane == 0) {
+        s_box[d][warp] = lo[d];
+        s_box[3 + d][warp] = hi[d];
+      }
+    }
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    {  // thread t: can any point of the box be within sample t's bound?  (FP32
+       // subtraction, max and dist2 are monotone, so no point that passes below is lost)
+      const float4 q = s_sample[threadIdx.x];
+      float bl[3], bh[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        bl[d] = s_box[d][0];
+        bh[d] = s_box[3 + d][0];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) {
+          bl[d] = fminf(bl[d], s_box[d][w]);
+          bh[d] = fmaxf(bh[d], s_box[3 + d][w]);
+        }
+      }
+      const float dx = fmaxf(fmaxf(bl[0] - q.x, q.x - bh[0]), 0.0f);
+      const float dy = fmaxf(fmaxf(bl[1] - q.y, q.y - bh[1]), 0.0f);
+      const float dz = fmaxf(fmaxf(bl[2] - q.z, q.z - bh[2]), 0.0f);
+      if (dist2(dx, dy, dz) <= q.w) s_pick[atomicAdd(&s_n, 1)] = threadIdx.x;
+    }
+    __syncthreads();
+    const int picked = s_n;
+    for (int r = 0; r < picked; ++r) {
+      const int t = s_pick[r];
+      const float4 q = s_sample[t];
+      float d2[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) d2[u] = dist2(x[u] - q.x, y[u] - q.y, z[u] - q.z);
+      if (!(fminf(fminf(d2[0], d2[1]), fminf(d2[2], d2[3])) <= q.w)) continue;
+      const int64_t si = sample_index(t, n);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t j = t0 + u * 256 + threadIdx.x;
+        if (d2[u] <= q.w && j < n && j != si) {
+          const uint32_t slot = atomicAdd(list_count + t, 1u);
+          if (slot < kListCap) list[(size_t)t * kListCap + slot] = d2[u];
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// out[s] = the k-NN distance of sample s.  scanned: whether k_sample_scan ran
+// (else the bound came from the whole cloud).
+__global__ void __launch_bounds__(256) k_sample_select(const float* __restrict__ xyz, int64_t n, int k, int scanned,
+                                                       const float* __restrict__ bound,
+                                                       const uint32_t* __restrict__ list_count,
+                                                       const float* __restrict__ list, float* out) {
+  float kth = bound[blockIdx.x];
+  if (scanned) {
+    const uint32_t count = list_count[blockIdx.x];
+    float best[kMaxK];
+    int m = 0;
+    if (count <= kListCap) {
+      for (uint32_t j = threadIdx.x; j < count; j += blockDim.x)
+        insert_k(best, k, m, list[(size_t)blockIdx.x * kListCap + j]);
+    } else {
+      const int64_t si = sample_index(blockIdx.x, n);
+      const float px = __ldg(xyz + 3 * si), py = __ldg(xyz + 3 * si + 1), pz = __ldg(xyz + 3 * si + 2);
+      for (int64_t j = threadIdx.x; j < n; j += blockDim.x)
+        if (j != si)
+          insert_k(best, k, m, dist2(__ldg(xyz + 3 * j) - px, __ldg(xyz + 3 * j + 1) - py, __ldg(xyz + 3 * j + 2) - pz));
+    }
+    __syncwarp();
+    kth = block_kth(best, k, m);
+  }
+  if (threadIdx.x == 0) out[blockIdx.x] = sqrtf(kth);
+}
+
+// Two grids over the bounding box: cells of h, which bound how far a search
+// goes, and search cells of kSearch h, which hold the sorted points.
 struct Grid {
-  float ox, oy, oz, inv_h, h;
-  uint32_t mask;  // buckets - 1
+  float ox, oy, oz;
+  float inv_h, inv_s;  // 1 / h, 1 / (kSearch h)
+  float s2_low;        // (kSearch h)^2, a little less: squared distances in search cells times this are lower bounds
+  float slack;         // in search cells: the rounding of two points' cell coordinates
+  uint32_t mask;       // buckets - 1
 };
 
-__device__ __forceinline__ void cell_of(const Grid& g, float x, float y, float z, int& cx, int& cy, int& cz) {
-  cx = (int)floorf((x - g.ox) * g.inv_h);
-  cy = (int)floorf((y - g.oy) * g.inv_h);
-  cz = (int)floorf((z - g.oz) * g.inv_h);
+__device__ __forceinline__ void cell_of(const Grid& g, float inv, float x, float y, float z, int& cx, int& cy, int& cz) {
+  cx = (int)floorf((x - g.ox) * inv);
+  cy = (int)floorf((y - g.oy) * inv);
+  cz = (int)floorf((z - g.oz) * inv);
 }
 
-__device__ __forceinline__ uint32_t bucket(const Grid& g, int cx, int cy, int cz) {
-  return (((uint32_t)cx * 73856093u) ^ ((uint32_t)cy * 19349663u) ^ ((uint32_t)cz * 83492791u)) & g.mask;
+// Bucket of a search cell: a multiplicative hash with the first rounds of
+// murmur3's 32-bit finalizer, so that the few occupied cells of a surface
+// spread over the table.
+__device__ __forceinline__ uint32_t bucket(const Grid& g, int Cx, int Cy, int Cz) {
+  uint32_t v = ((uint32_t)Cx * 73856093u) ^ ((uint32_t)Cy * 19349663u) ^ ((uint32_t)Cz * 83492791u);
+  v ^= v >> 16;
+  v *= 0x85ebca6bu;
+  v ^= v >> 13;
+  return v & g.mask;
 }
 
-__global__ void k_count(const float* __restrict__ xyz, int64_t n, Grid g, uint32_t* __restrict__ bkt,
-                        uint32_t* __restrict__ count) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    int cx, cy, cz;
-    cell_of(g, __ldg(xyz + 3 * i), __ldg(xyz + 3 * i + 1), __ldg(xyz + 3 * i + 2), cx, cy, cz);
-    const uint32_t b = bucket(g, cx, cy, cz);
-    bkt[i] = b;
-    atomicAdd(count + b, 1u);
+// Tells apart the cells that share a bucket.  Two cells of one search (at most
+// 14 apart along an axis) never have the same tag, so no point is met twice; a
+// distant point with the same tag and bucket is met as the distant point that
+// it is.
+__device__ __forceinline__ uint32_t cell_tag(int Cx, int Cy, int Cz) {
+  return (uint32_t)Cx + ((uint32_t)Cy << 10) + ((uint32_t)Cz << 20);
+}
+
+// Counts every bucket and keeps the count's old value, the point's rank in
+// its bucket, so that the scatter needs no atomics.  Four points a thread, so
+// that their round trips overlap.
+constexpr int kAhead = 4;
+
+__global__ void __launch_bounds__(256) k_count(const float* __restrict__ xyz, int64_t n, Grid g,
+                                               uint2* __restrict__ bkt, uint32_t* __restrict__ count) {
+  const int64_t S = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kAhead * S) {
+    uint32_t b[kAhead], rank[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int64_t i = min(i0 + u * S, n - 1);
+      int cx, cy, cz;
+      cell_of(g, g.inv_s, __ldg(xyz + 3 * i), __ldg(xyz + 3 * i + 1), __ldg(xyz + 3 * i + 2), cx, cy, cz);
+      b[u] = bucket(g, cx, cy, cz);
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (i0 + u * S < n) rank[u] = atomicAdd(count + b[u], 1u);
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (i0 + u * S < n) bkt[i0 + u * S] = make_uint2(b[u], rank[u]);
   }
 }
 
@@ -179,7 +406,7 @@ __global__ void __launch_bounds__(1024) k_scan_sums(uint32_t* __restrict__ tile_
 
 __global__ void __launch_bounds__(1024) k_scan_apply(const uint32_t* __restrict__ count, int64_t m,
                                                      const uint32_t* __restrict__ tile_off, uint32_t* __restrict__ start,
-                                                     uint32_t* __restrict__ cursor, uint32_t total) {
+                                                     uint32_t total) {
   __shared__ uint32_t warp_sum[32];
   const int64_t t0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * 4;
   uint32_t v[4], s = 0;
@@ -210,91 +437,255 @@ __global__ void __launch_bounds__(1024) k_scan_apply(const uint32_t* __restrict_
   for (int q = 0; q < 4; ++q)
     if (t0 + q < m) {
       start[t0 + q] = run;
-      cursor[t0 + q] = run;
       run += v[q];
     }
   if (blockIdx.x == 0 && threadIdx.x == 0) start[m] = total;
 }
 
-__global__ void k_scatter(const float* __restrict__ xyz, int64_t n, const uint32_t* __restrict__ bkt,
-                          uint32_t* __restrict__ cursor, float4* __restrict__ sorted) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t pos = atomicAdd(cursor + bkt[i], 1u);
-    sorted[pos] = make_float4(__ldg(xyz + 3 * i), __ldg(xyz + 3 * i + 1), __ldg(xyz + 3 * i + 2),
-                              __int_as_float((int)i));
+__global__ void __launch_bounds__(256) k_scatter(const float* __restrict__ xyz, int64_t n, Grid g,
+                                                 const uint2* __restrict__ bkt, const uint32_t* __restrict__ start,
+                                                 float4* __restrict__ sorted, uint32_t* __restrict__ index) {
+  const int64_t S = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kAhead * S) {
+    uint2 b[kAhead];
+    float4 p[kAhead];
+    uint32_t pos[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int64_t i = min(i0 + u * S, n - 1);
+      b[u] = __ldg(bkt + i);
+      p[u].x = __ldg(xyz + 3 * i);
+      p[u].y = __ldg(xyz + 3 * i + 1);
+      p[u].z = __ldg(xyz + 3 * i + 2);
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) pos[u] = __ldg(start + b[u].x) + b[u].y;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      if (i0 + u * S >= n) continue;
+      int cx, cy, cz;
+      cell_of(g, g.inv_s, p[u].x, p[u].y, p[u].z, cx, cy, cz);
+      p[u].w = __uint_as_float(cell_tag(cx, cy, cz));
+      sorted[pos[u]] = p[u];
+      index[pos[u]] = (uint32_t)(i0 + u * S);
+    }
   }
 }
 
-// Work per point is bounded: at most kMaxRing shells and kMaxScan candidate
-// points.  Within those limits the result is exact; past them the point gets
-// the k-th smallest distance found so far (an upper bound, and the true value
-// is then at least kMaxRing cells away), or +inf if fewer than k were found.
+// The search is bounded: a point's result is the k-th smallest distance to
+// the points at most kMaxRing cells away along each axis (+inf if there are
+// fewer than k) -- the exact result unless the true neighbour is further than
+// that, else an upper bound -- and at most kMaxScan candidates are looked at
+// (a cell with more copies of one place than that), past which the k-th
+// smallest found so far stands.
 constexpr int kMaxRing = 8;
 constexpr int kMaxScan = 1 << 16;
 
-__global__ void __launch_bounds__(256) k_query(const float* __restrict__ xyz, int64_t n, int k, Grid g,
-                                               const uint32_t* __restrict__ start, const float4* __restrict__ sorted,
-                                               int max_ring, float* __restrict__ radius) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float px = __ldg(xyz + 3 * i), py = __ldg(xyz + 3 * i + 1), pz = __ldg(xyz + 3 * i + 2);
-    int cx, cy, cz;
-    cell_of(g, px, py, pz, cx, cy, cz);
-    float best[kMaxK];
-    int m = 0, scanned = 0;
-    bool done = false;
-    const int rings = min(max_ring, kMaxRing);
-    for (int r = 0; r <= rings && !done; ++r) {
-      for (int dz = -r; dz <= r && !done; ++dz)
-        for (int dy = -r; dy <= r && !done; ++dy)
-          for (int dx = -r; dx <= r && !done; ++dx) {
-            if (max(abs(dx), max(abs(dy), abs(dz))) != r) continue;  // this shell only
-            const int qx = cx + dx, qy = cy + dy, qz = cz + dz;
-            const uint32_t b = bucket(g, qx, qy, qz);
-            const uint32_t e = __ldg(start + b + 1);
-            for (uint32_t s = __ldg(start + b); s < e; ++s) {
-              if (++scanned > kMaxScan) {
-                done = true;
-                break;
-              }
-              const float4 q = __ldg(sorted + s);
-              if (__float_as_int(q.w) == (int)i) continue;
-              int ox, oy, oz;
-              cell_of(g, q.x, q.y, q.z, ox, oy, oz);
-              if (ox != qx || oy != qy || oz != qz) continue;  // another cell in the same bucket
-              const float ddx = q.x - px, ddy = q.y - py, ddz = q.z - pz;
-              insert_k(best, k, m, ddx * ddx + ddy * ddy + ddz * ddz);
-            }
-            if (m == k && best[k - 1] == 0.0f) done = true;  // k duplicates: nothing is closer
-          }
-      // every point outside the visited cube is at least r h away (minus rounding)
-      const float reach = (float)r * g.h * (1.0f - 1e-5f);
-      done = done || ((m == k) && best[k - 1] <= reach * reach);
+// The K smallest squared distances met, ascending; +inf where there are fewer.
+template <int K>
+struct Nearest {
+  float d[K];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int q = 0; q < K; ++q) d[q] = INFINITY;
+  }
+  __device__ __forceinline__ void insert(float v) {  // v < d[K - 1]
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      const float lo = fminf(d[q], v);
+      v = fmaxf(d[q], v);
+      d[q] = lo;
     }
-    radius[i] = m < k ? INFINITY : sqrtf(best[k - 1]);
+  }
+  // the k-th smallest, k <= K (K = 4 serves k = 4 alone, so that d stays in registers)
+  __device__ __forceinline__ float kth(int k) const { return K == 4 ? d[3] : d[k - 1]; }
+};
+
+// One thread per point, in sorted order, so that the lanes of a warp look at
+// the same buckets.  A point looks at the 2 x 2 x 2 search cells nearest to it:
+// its own and the neighbours on the nearer side of each axis, so everything
+// nearer than half a search cell, and up to a whole one, is among them.  The
+// non-empty ranges go to shared memory first and the candidates of all of
+// them form one loop: with a loop per cell a warp ran the longest range of its
+// lanes eight times over (983 us on 5M points under ncu, 76% issue active; now
+// 781 us).  Bound by instruction issue and, the candidates of a warp lying in
+// several cells, by the L1: 32 KB of ranges a block instead of 16 cost it its
+// L1 share and 1050 us, 40 registers (6 blocks per SM) 900 us.  Search cells of 1.6 h: 38
+// candidates a point on a jittered surface; 2 h: 60, 1.25 h: 24 but 23% of the
+// points unsettled.  The unsettled ones are listed for k_query_far with their
+// distance so far in radius.  K = 4 (in registers) for k = 4, else 16.
+constexpr float kSearch = 1.6f;
+
+template <int K>
+__global__ void __launch_bounds__(256) k_query(int64_t n, int k, Grid g, const uint32_t* __restrict__ start,
+                                               const float4* __restrict__ sorted,
+                                               const uint32_t* __restrict__ index, float* __restrict__ radius,
+                                               uint32_t* __restrict__ pending, uint32_t* __restrict__ pending_count) {
+  __shared__ uint2 s_range[8][256];  // first point, count and octant
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const float4 p = __ldg(sorted + i);
+    int cx, cy, cz;
+    cell_of(g, g.inv_s, p.x, p.y, p.z, cx, cy, cz);
+    // per axis: the nearer neighbour, and the distance to it in search cells
+    const float ux = (p.x - g.ox) * g.inv_s - (float)cx, uy = (p.y - g.oy) * g.inv_s - (float)cy,
+                uz = (p.z - g.oz) * g.inv_s - (float)cz;
+    const int sx = ux < 0.5f ? -1 : 1, sy = uy < 0.5f ? -1 : 1, sz = uz < 0.5f ? -1 : 1;
+    const float near = fmaxf(fminf(ux, 1.0f - ux), fmaxf(fminf(uy, 1.0f - uy), fminf(uz, 1.0f - uz)));
+    int ranges = 0, scanned = 0;
+    uint32_t rs[8], re[8];
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {  // own cell first
+      const uint32_t b = bucket(g, cx + ((o & 1) ? sx : 0), cy + ((o & 2) ? sy : 0), cz + ((o & 4) ? sz : 0));
+      rs[o] = __ldg(start + b);
+      re[o] = __ldg(start + b + 1);
+    }
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+      const int len = (int)min(re[o] - rs[o], (uint32_t)(kMaxScan - scanned));
+      if (len > 0)
+        s_range[ranges++][threadIdx.x] = make_uint2(rs[o], (uint32_t)len | ((uint32_t)o << 20));
+      scanned += len;
+    }
+    Nearest<K> best;
+    best.clear();
+    uint32_t s = 0, e = 0, tag = 0;
+    const uint32_t own_tag = cell_tag(cx, cy, cz), tx = (uint32_t)sx, ty = (uint32_t)sy << 10, tz = (uint32_t)sz << 20;
+    for (int r = 0;;) {
+      if (s == e) {
+        if (r == ranges || best.kth(k) == 0.0f) break;  // (k copies: nothing is closer)
+        const uint2 v = s_range[r++][threadIdx.x];
+        s = v.x;
+        e = s + (v.y & 0xfffffu);
+        tag = own_tag + ((v.y >> 20) & 1u) * tx + ((v.y >> 21) & 1u) * ty + (v.y >> 22) * tz;
+      }
+      const float4 q = __ldg(sorted + s);
+      const float d2 = dist2(q.x - p.x, q.y - p.y, q.z - p.z);
+      best.insert((__float_as_uint(q.w) == tag && s != (uint32_t)i) ? d2 : INFINITY);
+      ++s;
+    }
+    const float kth = best.kth(k);
+    const float reach = fmaxf(1.0f - near - g.slack, 0.0f);
+    radius[__ldg(index + i)] = sqrtf(kth);
+    if (kth > reach * reach * g.s2_low && scanned < kMaxScan) pending[atomicAdd(pending_count, 1u)] = (uint32_t)i;
+  }
+}
+
+// The points that their nearest cells did not settle (1 in 100 of a jittered
+// surface), a warp each, a cell a lane: the cells that a ball around the point
+// meets, its radius the distance found so far (every nearer point is in it),
+// or 4 h and 9 h (past which nothing counts) while fewer than k points were
+// found.  (A thread each took 188 us on 5M points: few threads, each a chain
+// of some 27 lookups.)
+template <int K>
+__global__ void __launch_bounds__(256) k_query_far(int k, Grid g, const uint32_t* __restrict__ start,
+                                                   const float4* __restrict__ sorted,
+                                                   const uint32_t* __restrict__ index, int max_ring,
+                                                   float* __restrict__ radius, const uint32_t* __restrict__ pending,
+                                                   const uint32_t* __restrict__ pending_count) {
+  const uint32_t count = *pending_count;
+  const int rings = min(max_ring, kMaxRing);
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < count; j += warps) {  // warp-uniform
+    const uint32_t i = pending[j];
+    const float4 p = __ldg(sorted + i);
+    const uint32_t at = __ldg(index + i);
+    int cx, cy, cz;
+    cell_of(g, g.inv_h, p.x, p.y, p.z, cx, cy, cz);
+    const float fx = (p.x - g.ox) * g.inv_s, fy = (p.y - g.oy) * g.inv_s, fz = (p.z - g.oz) * g.inv_s;
+    float found = radius[at];  // an upper bound of the result, or +inf
+    const float most = (float)(rings + 1) / kSearch + g.slack;  // search cells that the cube of +-rings cells spans
+    bool last;
+    float ball = 0.0f;
+    do {
+      if (found < INFINITY) {
+        ball = fminf(found * g.inv_s * 1.00001f + g.slack, most);
+        last = true;
+      } else {
+        ball = ball == 0.0f ? fminf(4.0f / kSearch, most) : most;
+        last = ball == most;
+      }
+      const float limit = found < INFINITY ? found * found * 1.00001f : INFINITY;
+      Nearest<K> best;
+      best.clear();
+      int scanned = 0;
+      const int x0 = (int)floorf(fx - ball), y0 = (int)floorf(fy - ball), z0 = (int)floorf(fz - ball);
+      const int nx = (int)floorf(fx + ball) - x0 + 1, ny = (int)floorf(fy + ball) - y0 + 1,
+                nz = (int)floorf(fz + ball) - z0 + 1;
+      for (int c = lane; c < nx * ny * nz && scanned < kMaxScan; c += 32) {
+        const int qx = x0 + c % nx, qy = y0 + c / nx % ny, qz = z0 + c / (nx * ny);
+        const float dx = fmaxf(fmaxf((float)qx - fx, fx - (float)(qx + 1)) - g.slack, 0.0f);
+        const float dy = fmaxf(fmaxf((float)qy - fy, fy - (float)(qy + 1)) - g.slack, 0.0f);
+        const float dz = fmaxf(fmaxf((float)qz - fz, fz - (float)(qz + 1)) - g.slack, 0.0f);
+        if ((dx * dx + dy * dy + dz * dz) * g.s2_low > limit) continue;
+        const uint32_t b = bucket(g, qx, qy, qz), tag = cell_tag(qx, qy, qz);
+        uint32_t s = __ldg(start + b);
+        const uint32_t e = s + min(__ldg(start + b + 1) - s, (uint32_t)(kMaxScan - scanned));
+        scanned += (int)(e - s);
+        for (; s < e; ++s) {
+          const float4 q = __ldg(sorted + s);
+          const float d2 = dist2(q.x - p.x, q.y - p.y, q.z - p.z);
+          if (!(d2 < best.d[K - 1]) || __float_as_uint(q.w) != tag || s == i) continue;
+          int ox, oy, oz;  // the cube of +-rings cells bounds what counts
+          cell_of(g, g.inv_h, q.x, q.y, q.z, ox, oy, oz);
+          if (max(abs(ox - cx), max(abs(oy - cy), abs(oz - cz))) <= rings) best.insert(d2);
+        }
+      }
+      __syncwarp();
+      // the k-th smallest of the lanes' lists: k times the least head
+      float kth = INFINITY;
+      for (int r = 0; r < k; ++r) {  // (distances are >= 0: their bits order as they do)
+        const uint32_t head = __float_as_uint(best.d[0]);
+        const uint32_t least = __reduce_min_sync(0xffffffffu, head);
+        const unsigned who = __ballot_sync(0xffffffffu, head == least);
+        if (lane == __ffs(who) - 1) {
+#pragma unroll
+          for (int q = 0; q < K - 1; ++q) best.d[q] = best.d[q + 1];
+          best.d[K - 1] = INFINITY;
+        }
+        kth = __uint_as_float(least);
+      }
+      found = sqrtf(kth);
+      // the k-th of a first, smaller ball is exact if the ball reaches it
+      if (found < INFINITY && found * g.inv_s * 1.00001f + g.slack <= ball) last = true;
+      if (__any_sync(0xffffffffu, scanned >= kMaxScan)) last = true;
+    } while (!last);
+    if (lane == 0) radius[at] = found;
   }
 }
 
 struct Layout {
-  size_t box, samples, bkt, count, start, cursor, tiles, sorted, total;
-  int64_t m;
+  size_t box, samples, bound, list_count, list, bkt, count, start, tiles, sorted, index, pending, total;
+  int64_t m;            // buckets
+  int64_t groups;       // groups of kSubGroup points in the samples' subset
+  bool scan;            // the subset is not the whole cloud
 };
 
 size_t up(size_t v) { return (v + 255) / 256 * 256; }
 
 Layout layout(int64_t n) {
   Layout L{};
-  int64_t m = 1;
-  while (m < n) m <<= 1;
+  // in the median a search cell holds 4 (curves), 9 (surfaces) or 12 (volumes) points
+  int64_t m = 256;
+  while (m < n / 4) m <<= 1;
   L.m = m;
+  const int64_t total = (n + kSubGroup - 1) / kSubGroup;
+  L.groups = std::min(total, std::max((int64_t)kSubLeast / kSubGroup, total / 128));
+  L.scan = L.groups < total;
   size_t o = 0;
-  L.box = o;       o = up(o + 6 * 4);
-  L.samples = o;   o = up(o + kSamples * 4);
-  L.bkt = o;       o = up(o + (size_t)n * 4);
-  L.count = o;     o = up(o + (size_t)m * 4);
-  L.start = o;     o = up(o + ((size_t)m + 1) * 4);
-  L.cursor = o;    o = up(o + (size_t)m * 4);
-  L.tiles = o;     o = up(o + (size_t)((m + kScanTile - 1) / kScanTile) * 4);
-  L.sorted = o;    o = up(o + (size_t)n * 16);
+  L.box = o;         o = up(o + 7 * 4);  // and the count of pending
+  L.samples = o;     o = up(o + kSamples * 4);
+  L.bound = o;       o = up(o + kSamples * 4);
+  L.list_count = o;  o = up(o + kSamples * 4);
+  L.list = o;        o = up(o + (L.scan ? (size_t)kSamples * kListCap * 4 : 0));
+  L.bkt = o;         o = up(o + (size_t)n * 8);
+  L.count = o;       o = up(o + (size_t)m * 4);
+  L.start = o;       o = up(o + ((size_t)m + 1) * 4);
+  L.tiles = o;       o = up(o + (size_t)((m + kScanTile - 1) / kScanTile) * 4);
+  L.sorted = o;      o = up(o + (size_t)n * 16);
+  L.index = o;       o = up(o + (size_t)n * 4);
+  L.pending = o;     o = up(o + (size_t)n * 4);
   L.total = o;
   return L;
 }
@@ -330,19 +721,26 @@ adop_status adop_point_radius(const float* xyz, int64_t n, int32_t k, float* rad
   char* ws = static_cast<char*>(workspace);
   uint32_t* box = reinterpret_cast<uint32_t*>(ws + L.box);
   float* samples = reinterpret_cast<float*>(ws + L.samples);
-  uint32_t* bkt = reinterpret_cast<uint32_t*>(ws + L.bkt);
+  float* bound = reinterpret_cast<float*>(ws + L.bound);
+  uint32_t* list_count = reinterpret_cast<uint32_t*>(ws + L.list_count);
+  float* list = reinterpret_cast<float*>(ws + L.list);
+  uint2* bkt = reinterpret_cast<uint2*>(ws + L.bkt);
   uint32_t* count = reinterpret_cast<uint32_t*>(ws + L.count);
   uint32_t* start = reinterpret_cast<uint32_t*>(ws + L.start);
-  uint32_t* cursor = reinterpret_cast<uint32_t*>(ws + L.cursor);
   uint32_t* tiles = reinterpret_cast<uint32_t*>(ws + L.tiles);
   float4* sorted = reinterpret_cast<float4*>(ws + L.sorted);
+  uint32_t* index = reinterpret_cast<uint32_t*>(ws + L.index);
+  uint32_t* pending = reinterpret_cast<uint32_t*>(ws + L.pending);
   const int blocks = adop::num_sms() * 8;
   cudaError_t e;
-  const uint32_t init[6] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
-  if ((e = cudaMemcpyAsync(box, init, sizeof(init), cudaMemcpyHostToDevice, s)) != cudaSuccess)
+  if ((e = cudaMemsetAsync(box, 0xff, 3 * 4, s)) != cudaSuccess ||
+      (e = cudaMemsetAsync(box + 3, 0, 4 * 4, s)) != cudaSuccess)
     return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   k_bbox<<<blocks, 256, 0, s>>>(xyz, n, box);
-  k_sample_knn<<<kSamples, 256, 0, s>>>(xyz, n, k, samples);
+  k_sample_bound<<<kSamples, kBoundThreads, 0, s>>>(xyz, n, k, L.groups, bound, list_count);
+  if (L.scan)
+    k_sample_scan<<<(unsigned)std::min((n + 1023) / 1024, (int64_t)blocks), 256, 0, s>>>(xyz, n, bound, list_count, list);
+  k_sample_select<<<kSamples, 256, 0, s>>>(xyz, n, k, L.scan ? 1 : 0, bound, list_count, list, samples);
   uint32_t hbox[6];
   float hs[kSamples];
   if ((e = cudaMemcpyAsync(hbox, box, sizeof(hbox), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
@@ -374,15 +772,25 @@ adop_status adop_point_radius(const float* xyz, int64_t n, int32_t k, float* rad
   h = std::max({h, extent / 1048576.0f, 1e-20f});
   if (v.empty()) h = std::max(extent, 1e-20f);  // fewer than k + 1 points
   const int max_ring = (int)std::ceil(extent / h) + 2;
-  Grid g{lo[0], lo[1], lo[2], 1.0f / h, h, (uint32_t)(L.m - 1)};
+  const float cell = h * kSearch;
+  const Grid g{lo[0], lo[1], lo[2], 1.0f / h, 1.0f / cell, cell * cell * 0.99998f, extent / cell * 5e-7f + 1e-6f,
+               (uint32_t)(L.m - 1)};
   if ((e = cudaMemsetAsync(count, 0, (size_t)L.m * 4, s)) != cudaSuccess) return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   k_count<<<blocks, 256, 0, s>>>(xyz, n, g, bkt, count);
   const int64_t nt = (L.m + kScanTile - 1) / kScanTile;
   k_scan_tiles<<<(unsigned)nt, 1024, 0, s>>>(count, L.m, tiles);
   k_scan_sums<<<1, 1024, 0, s>>>(tiles, nt);
-  k_scan_apply<<<(unsigned)nt, 1024, 0, s>>>(count, L.m, tiles, start, cursor, (uint32_t)n);
-  k_scatter<<<blocks, 256, 0, s>>>(xyz, n, bkt, cursor, sorted);
-  k_query<<<blocks, 256, 0, s>>>(xyz, n, k, g, start, sorted, max_ring, radius);
+  k_scan_apply<<<(unsigned)nt, 1024, 0, s>>>(count, L.m, tiles, start, (uint32_t)n);
+  k_scatter<<<blocks, 256, 0, s>>>(xyz, n, g, bkt, start, sorted, index);
+  const unsigned qblocks = (unsigned)std::min((n + 255) / 256, (int64_t)blocks * 8);
+  uint32_t* pending_count = box + 6;
+  if (k == 4) {
+    k_query<4><<<qblocks, 256, 0, s>>>(n, k, g, start, sorted, index, radius, pending, pending_count);
+    k_query_far<4><<<blocks, 256, 0, s>>>(k, g, start, sorted, index, max_ring, radius, pending, pending_count);
+  } else {
+    k_query<kMaxK><<<qblocks, 256, 0, s>>>(n, k, g, start, sorted, index, radius, pending, pending_count);
+    k_query_far<kMaxK><<<blocks, 256, 0, s>>>(k, g, start, sorted, index, max_ring, radius, pending, pending_count);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   return ADOP_OK;
 }
