@@ -254,6 +254,7 @@ void fill_cam(DevCam& d, const adop_camera& cam, const adop_frame* f, bool use_f
     d.image[l] = f ? f->image[l] : nullptr;
   }
   d.acc = use_frame_state ? f->acc : reinterpret_cast<float*>(ws + L.acc[k]);
+  d.keep_acc = use_frame_state ? 1 : 0;
   d.vis = use_frame_state ? f->vis : reinterpret_cast<uint32_t*>(ws + L.vis[k]);
   d.early = reinterpret_cast<uint8_t*>(ws + L.early[k]);
   d.info = reinterpret_cast<float*>(ws + L.info[k]);
@@ -308,15 +309,21 @@ adop_status render_chunk(const adop_points* pts, const adop_camera* cams, int k0
     const int k = k0 + j;
     const bool use_frame = frames_state && state_given(frames[k], prm->levels) == 1;
     fill_cam(lc.c[j], cams[k], frames ? &frames[k] : nullptr, use_frame, L, k, ws, pts, prm);
+    // without kept state nothing reads the layer masks (a backward renders
+    // again, and records them then): 4 bytes a point and camera not written
+    if (!use_frame) lc.c[j].vis = nullptr;
     if (!normalize)
       for (int l = 0; l < ADOP_MAX_LEVELS; ++l) lc.c[j].image[l] = nullptr;
   }
-  const PointArgs a = point_args(pts, prm, nc);
+  PointArgs a = point_args(pts, prm, nc);
+  a.seeded = seed_rule(lc, a, pts->c);
   cudaError_t e;
   if ((e = timed("clear", s, [&] { return launch_clear(lc, a, pts->c, s); })) != cudaSuccess)
     return cuda_fail(e, "clear launch");
   if ((e = timed("depth", s, [&] { return launch_depth(lc, a, s); })) != cudaSuccess)
     return cuda_fail(e, "depth pass launch");
+  if ((e = timed("seed", s, [&] { return launch_seed(lc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
+    return cuda_fail(e, "seed launch");
   if ((e = timed("accumulate", s, [&] { return launch_accum(lc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
     return cuda_fail(e, "accumulate launch");
   if (normalize) {
@@ -563,11 +570,14 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
         if (state_given(frames[k0 + j], params->levels) == 0) idx[m++] = k0 + j;
       if (m > 0) {
         for (int j = 0; j < m; ++j) fill_cam(rc.c[j], cams[idx[j]], nullptr, false, L, idx[j], ws, pts, params);
-        const PointArgs a = point_args(pts, params, m);
+        PointArgs a = point_args(pts, params, m);
+        a.seeded = seed_rule(rc, a, pts->c);
         if ((e = timed("clear", s, [&] { return launch_clear(rc, a, pts->c, s); })) != cudaSuccess)
           return cuda_fail(e, "clear launch");
         if ((e = timed("depth", s, [&] { return launch_depth(rc, a, s); })) != cudaSuccess)
           return cuda_fail(e, "depth pass launch");
+        if ((e = timed("seed", s, [&] { return launch_seed(rc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
+          return cuda_fail(e, "seed launch");
         if ((e = timed("accumulate", s, [&] { return launch_accum(rc, a, pts->c, pts->feat_dtype, s); })) !=
             cudaSuccess)
           return cuda_fail(e, "accumulate launch");

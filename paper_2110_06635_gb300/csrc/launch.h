@@ -78,6 +78,7 @@ struct PointArgs {
   float znear;
   float a1;             // f32(1 + alpha)
   uint32_t flags;
+  int32_t seeded;       // the forward's sums start from the pixels' nearest points (seed_rule)
   int32_t grad_dtype;   // adop_dtype of the upstream gradients (DevCam::grad)
 };
 
@@ -115,8 +116,11 @@ int64_t most_points(const LaunchCams& cams, const PointArgs& a);
 // 72 -> 64 us and accumulate 100 -> 91 us at unchanged DRAM traffic and L2
 // hit rate; more waves than these were slower again.)
 constexpr int kPointWaves = 10;  // k_depth, k_accum
-constexpr int kPixelWaves = 6;   // k_clear, k_normalize, k_bwd_prepass, k_env_*
-dim3 stride_grid(const void* k, int64_t work, int ncam, int waves, size_t smem);
+constexpr int kPixelWaves = 6;   // k_clear, k_seed, k_normalize, k_bwd_prepass, k_env_*
+dim3 stride_grid(const void* k, int64_t work, int ncam, int waves, size_t smem, int threads = kThreads);
+
+// Whether the forward of these cameras seeds its sums (PointArgs::seeded).
+int seed_rule(const LaunchCams& cams, const PointArgs& a, int c);
 
 // launch_pdl of a grid-stride kernel over `work` items per camera, on the
 // stride_grid() of that kernel.
@@ -129,6 +133,7 @@ cudaError_t launch_strided(void (*k)(KArgs...), int64_t work, int ncam, int wave
 
 cudaError_t launch_clear(const LaunchCams& cams, const PointArgs& a, int c, cudaStream_t s);
 cudaError_t launch_depth(const LaunchCams& cams, const PointArgs& a, cudaStream_t s);
+cudaError_t launch_seed(const LaunchCams& cams, const PointArgs& a, int c, adop_dtype fd, cudaStream_t s);
 cudaError_t launch_accum(const LaunchCams& cams, const PointArgs& a, int c, adop_dtype fd, cudaStream_t s);
 cudaError_t launch_normalize(const LaunchCams& cams, const PointArgs& a, int c, adop_dtype od, cudaStream_t s);
 cudaError_t launch_bwd_prepass(const LaunchCams& cams, const PointArgs& a, int c, cudaStream_t s);

@@ -220,8 +220,10 @@ void Server::launch_locked() {
     a.flags = cfg.flags;
     cudaStream_t st = streams[s];
     const PdlScope pdl(pdl_for_points(a.n, a.ncam));
+    a.seeded = adop::seed_rule(lc, a, c);
     cudaError_t e = launch_clear(lc, a, c, st);
     if (e == cudaSuccess) e = launch_depth(lc, a, st);
+    if (e == cudaSuccess) e = launch_seed(lc, a, c, feat_dtype, st);
     if (e == cudaSuccess) e = launch_accum(lc, a, c, feat_dtype, st);
     if (e == cudaSuccess) e = launch_normalize(lc, a, c, cfg.out_dtype, st);
     if (e == cudaSuccess && cfg.env) e = launch_env_fill(lc, a, c, cfg.out_dtype, st);

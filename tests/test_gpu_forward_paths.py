@@ -1,0 +1,60 @@
+"""The forward's launch-time choices against the oracle: sums seeded with each
+pixel's nearest point (from 96 MB of pixel state) or cleared, one or four
+points a lane in the accumulate pass (from 311296 points on 152 SMs), every
+depth-pass layer count, state kept or rendered again by the backward, and a
+layer-mask buffer that is only 4-byte aligned."""
+import numpy as np
+import pytest
+
+import scenes
+from parity import compare, gpu_run, oracle_run
+
+pytestmark = pytest.mark.gpu
+
+
+def _camera(w, h, **kw):
+    return scenes.Camera(w, h, 0.9 * w, 0.9 * w, w / 2, h / 2, k1=0.01, R=np.eye(3, dtype=np.float32),
+                         t=np.array([-0.5, -0.5, 2.0], np.float32), **kw)
+
+
+@pytest.mark.parametrize("n,c,dtype,levels,w,h,keep", [
+    (311_295, 4, "f32", 4, 320, 200, True),     # one point a lane
+    (311_297, 4, "f32", 4, 320, 200, True),     # four, and a last chunk of one point
+    (400_003, 8, "bf16", 5, 333, 217, False),
+    (350_001, 2, "f16", 2, 320, 200, True),
+    (350_001, 1, "f32", 1, 320, 200, False),
+    (40_001, 8, "bf16", 4, 2200, 1500, True),   # seeded
+    (312_001, 8, "f32", 4, 2200, 1500, False),
+    (40_001, 16, "f16", 3, 1400, 1000, True),
+    (40_001, 3, "f32", 5, 2400, 2001, True),
+    (20_011, 1, "f32", 8, 3000, 2400, False)])
+def test_forward_and_backward_paths(adop, orc, n, c, dtype, levels, w, h, keep):
+    sc = scenes.tiny_spheres(n, c, seed=n % 1000)
+    cams = [_camera(w, h)]
+    G = [scenes.upstream_grad(w, h, levels, c, 7)]
+    g = gpu_run(adop, sc, cams, dtype, levels=levels, grads=G, keep_state=keep, grad_assign=True)
+    r = oracle_run(orc, sc, cams, dtype, levels=levels, grads=G)
+    compare(g, r, dtype, check_state=keep)
+    if keep:  # an empty pixel's sums are zero in a kept frame
+        fr = g["frames"][0]
+        acc = fr.acc.view(-1, c).cpu().numpy()
+        assert not acc[r["cnt"][0] == 0].any()
+
+
+def test_layer_masks_only_4_byte_aligned(adop):
+    import torch
+    sc = scenes.tiny_spheres(311_303, 4, seed=5)
+    cam = _camera(320, 200)
+    pts = adop.Points(torch.from_numpy(sc.xyz).cuda(), torch.from_numpy(sc.feat).cuda())
+    params = adop.Params(4, 0.01, 1e-3, None, 0)
+    got = []
+    for offset in (0, 1):
+        fr = adop.Frame.alloc(cam, 4, 4, torch.float32, True, "cuda", sc.n)
+        buf = torch.full((sc.n + 2,), -1, dtype=torch.int32, device="cuda")
+        fr.vis = buf[offset:offset + sc.n]
+        ws = adop.alloc_workspace(pts, [cam], params)
+        adop.adop_render_forward(pts, [cam], params, [fr], ws)
+        got.append(fr.vis.cpu().numpy())
+        assert buf[offset + sc.n] == -1 and (offset == 0 or buf[0] == -1)
+    assert np.array_equal(got[0], got[1])
+    assert (got[0] == 0).any() and (got[0] & 0xFF != 0).any()
