@@ -37,6 +37,7 @@ struct DevCam {
   float fx, fy, cx, cy, k1, k2, k3, p1, p2;
   float ifx, ify;  // f32(1 / fx), f32(1 / fy) (the inverse camera)
   int32_t w, h;
+  float inside_u, inside_v;  // -0.5 <= u0 < inside_u and v0 alike: inside the image at every layer
   int32_t model;  // 0 pinhole + Brown-Conrady, 1 fisheye (stereographic)
   int64_t off[ADOP_MAX_LEVELS + 1];  // first pixel of each layer in the concatenated pyramid
   unsigned long long* key[ADOP_MAX_LEVELS];
@@ -241,6 +242,24 @@ __device__ __forceinline__ bool camera(const DevCam& cam, float X0, float X1, fl
   return true;
 }
 
+// camera() for a pinhole without tangential terms, known when the kernel is
+// launched: the same operations without the tests.
+__host__ __device__ __forceinline__ bool camera_is_plain(const DevCam& cam) {
+  return cam.model == 0 && cam.p1 == 0.0f && cam.p2 == 0.0f;
+}
+__device__ __forceinline__ bool camera_plain(const DevCam& cam, float X0, float X1, float X2, float& u0, float& v0,
+                                             float& depth) {
+  depth = X2;
+  const float xn = __fdiv_rn(X0, X2);
+  const float yn = __fdiv_rn(X1, X2);
+  const float r2 = __fadd_rn(__fmul_rn(xn, xn), __fmul_rn(yn, yn));
+  const float d = __fadd_rn(
+      1.0f, __fmul_rn(r2, __fadd_rn(cam.k1, __fmul_rn(r2, __fadd_rn(cam.k2, __fmul_rn(r2, cam.k3))))));
+  u0 = __fadd_rn(__fmul_rn(cam.fx, __fmul_rn(xn, d)), cam.cx);
+  v0 = __fadd_rn(__fmul_rn(cam.fy, __fmul_rn(yn, d)), cam.cy);
+  return true;
+}
+
 // Eq. normalculling as printed: keep iff (R n)^T (R x + t) > 0.
 __device__ __forceinline__ bool normal_keep(const DevCam& cam, const float* nrm, int64_t i, float X0,
                                             float X1, float X2) {
@@ -275,9 +294,11 @@ __device__ __forceinline__ bool pixel_at(float u0, float v0, int l, int32_t w, i
 // integer test alone gives pixel_at's result.
 __device__ __forceinline__ bool pixel_in(float u0, float v0, int l, int32_t w, int32_t h, int32_t& pu,
                                          int32_t& pv) {
-  const float s = layer_scale(l);
-  pu = __float2int_rn(__fmul_rn(u0, s));
-  pv = __float2int_rn(__fmul_rn(v0, s));
+  // The addition of 1.5 2^23 rounds to the nearest integer, ties to even, for
+  // |u0 2^-l| < 2^22 (u0 2^-l itself is exact), and leaves it in the low bits.
+  const float s = layer_scale(l), m = 12582912.0f;
+  pu = __float_as_int(__fmaf_rn(u0, s, m)) - 0x4B400000;
+  pv = __float_as_int(__fmaf_rn(v0, s, m)) - 0x4B400000;
   return (uint32_t)pu < (uint32_t)(w >> l) && (uint32_t)pv < (uint32_t)(h >> l);
 }
 

@@ -391,6 +391,12 @@ void set_camera_constants(DevCam& d, const adop_camera& cam, int levels, uint32_
   d.h = cam.K.h;
   d.model = cam.K.model;
   pyramid_pixels(d.w, d.h, levels, d.off);
+  // layer l keeps u0 where rn(u0 2^-l) is in [0, w_l): from -0.5 (rounds to 0) to below (w_l - 0.5) 2^l
+  d.inside_u = d.inside_v = INFINITY;
+  for (int l = 0; l < levels; ++l) {
+    d.inside_u = std::fmin(d.inside_u, std::ldexp((float)(d.w >> l) - 0.5f, l));
+    d.inside_v = std::fmin(d.inside_v, std::ldexp((float)(d.h >> l) - 0.5f, l));
+  }
   d.tiles_x = tiles_along(d.w);
   d.tiles = d.tiles_x * tiles_along(d.h);
   const adop_photometric& ph = cam.ph;

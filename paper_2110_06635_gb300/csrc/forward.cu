@@ -108,43 +108,64 @@ __global__ void __launch_bounds__(kThreads) k_clear(const __grid_constant__ Laun
 // points are outside the view: accumulate 770 -> 581 us, and 528 us once the
 // position is read only for points with a layer left).
 // ---------------------------------------------------------------------------
-template <int kL>
+// One point at every layer.  kInside: the point is inside the image at every
+// layer (in_every_layer), so no layer is tested.  kPlain: no discarding.
+// Returns the layers where the point may still pass the fuzzy test.
+template <int kL, bool kInside, bool kPlain>
+__device__ __forceinline__ uint32_t depth_layers(const DevCam& cam, const PointArgs& a, float u0, float v0, float zd,
+                                                 uint32_t i) {
+  const bool discard = !kPlain && a.radius != nullptr;
+  const float rw = discard ? __ldg(a.radius + i) : 0.0f, bt = discard ? __ldg(a.beta + i) : 0.0f;
+  const int levels = kL < ADOP_MAX_LEVELS ? kL : a.levels;
+  int32_t pix[kL];  // pixel within layer l (< 2^28), -1: none
+#pragma unroll
+  for (int l = 0; l < kL; ++l) {
+    int32_t pu, pv;
+    const bool in = pixel_in(u0, v0, l, cam.w, cam.h, pu, pv);
+    pix[l] = pv * (cam.w >> l) + pu;
+    if (!(kInside || in) || l >= levels || (discard && !discard_keep(cam, zd, rw, bt, a.g2, l))) pix[l] = -1;
+  }
+  // Only the upper half of a key, the depth, is read.  (An L1-cached read may
+  // be stale, but keys only decrease: a stale value can cost an atomic that
+  // loses, never skip one that wins, and it can only keep a layer in the mask
+  // that a fresh value would have dropped.)
+  uint32_t cur[kL];
+#pragma unroll
+  for (int l = 0; l < kL; ++l)
+    cur[l] = pix[l] >= 0 ? __ldca(reinterpret_cast<const uint32_t*>(cam.key[l] + pix[l]) + 1) : 0u;
+  uint32_t em = 0;
+#pragma unroll
+  for (int l = 0; l < kL; ++l) {
+    // an empty pixel's depth reads as NaN, and nothing is behind it.  alpha >= 0:
+    // what is behind the fuzzy threshold is behind the nearest point too
+    if (pix[l] < 0 || zd > __fmul_rn(__uint_as_float(cur[l]), a.a1)) continue;
+    em |= 1u << l;
+    // (an equal depth may win by its index: the atomic decides)
+    if (__float_as_uint(zd) <= cur[l]) atomicMin(cam.key[l] + pix[l], depth_key(zd, i));
+  }
+  return em;
+}
+
+template <int kL, bool kPlain>
 __global__ void __launch_bounds__(kThreads) k_depth(const __grid_constant__ LaunchCams cams,
                                                     const __grid_constant__ PointArgs a) {
   pdl_entry();
   const DevCam& cam = cams.c[blockIdx.y];
   const float* __restrict__ xyz = cam.xyz;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cam.n; i += (int64_t)gridDim.x * blockDim.x) {
+  const uint32_t n = (uint32_t)cam.n, S = gridDim.x * blockDim.x;  // n < 2^31, S < 2^23: no wrap
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += S) {
+    const float* q = xyz + 3 * (int64_t)i;
     float X0, X1, X2, u0, v0, zd;
     uint32_t em = 0;  // layers where the point may still pass the fuzzy test
-    transform(cam, __ldg(xyz + 3 * i), __ldg(xyz + 3 * i + 1), __ldg(xyz + 3 * i + 2), X0, X1, X2);
-    if (camera(cam, X0, X1, X2, u0, v0, zd) && (zd > a.znear) && in_pyramid(u0, v0, cam.w, cam.h, a.levels) &&
-        !(cam.normals && !normal_keep(cam, cam.normals, i, X0, X1, X2))) {
-      const unsigned long long key = depth_key(zd, i);
-      const float rw = a.radius ? __ldg(a.radius + i) : 0.0f, bt = a.radius ? __ldg(a.beta + i) : 0.0f;
-      int32_t pix[kL];  // pixel within layer l (< 2^28), -1: none
-#pragma unroll
-      for (int l = 0; l < kL; ++l) {
-        int32_t pu, pv;
-        const bool keep = l < a.levels && (!a.radius || discard_keep(cam, zd, rw, bt, a.g2, l));
-        pix[l] = (keep && pixel_in(u0, v0, l, cam.w, cam.h, pu, pv)) ? pv * (cam.w >> l) + pu : -1;
-      }
-      // (an L1-cached read may be stale, but keys only decrease: a stale value
-      // can cost an atomic that loses, never skip one that wins, and it can
-      // only keep a layer in the mask that a fresh value would have dropped)
-      unsigned long long cur[kL];
-#pragma unroll
-      for (int l = 0; l < kL; ++l) cur[l] = pix[l] >= 0 ? __ldca(cam.key[l] + pix[l]) : 0ull;
-#pragma unroll
-      for (int l = 0; l < kL; ++l) {
-        if (pix[l] < 0) continue;
-        if (key < cur[l]) {
-          atomicMin(cam.key[l] + pix[l], key);
-          em |= 1u << l;
-        } else if (!(zd > __fmul_rn(__uint_as_float((uint32_t)(cur[l] >> 32)), a.a1))) {
-          em |= 1u << l;  // behind the current nearest point, but within the fuzzy threshold
-        }
-      }
+    transform(cam, __ldg(q), __ldg(q + 1), __ldg(q + 2), X0, X1, X2);
+    const bool ok = (kPlain ? camera_plain(cam, X0, X1, X2, u0, v0, zd) : camera(cam, X0, X1, X2, u0, v0, zd)) &&
+                    zd > a.znear;
+    if (ok && u0 >= -0.5f && u0 < cam.inside_u && v0 >= -0.5f && v0 < cam.inside_v) {
+      if (kPlain || !(cam.normals && !normal_keep(cam, cam.normals, i, X0, X1, X2)))
+        em = depth_layers<kL, true, kPlain>(cam, a, u0, v0, zd, i);
+    } else if (ok && in_pyramid(u0, v0, cam.w, cam.h, a.levels)) {
+      if (kPlain || !(cam.normals && !normal_keep(cam, cam.normals, i, X0, X1, X2)))
+        em = depth_layers<kL, false, kPlain>(cam, a, u0, v0, zd, i);
     }
     if (cam.early) __stcs(cam.early + i, (uint8_t)em);
   }
@@ -449,8 +470,20 @@ int64_t most_points(const LaunchCams& cams, const PointArgs& a) {
 cudaError_t launch_depth(const LaunchCams& cams, const PointArgs& a, cudaStream_t s) {
   const int64_t n = most_points(cams, a);
   if (n == 0) return cudaSuccess;
-  if (a.levels <= 4) return launch_strided(k_depth<4>, n, a.ncam, kPointWaves, 0, s, cams, a);
-  return launch_strided(k_depth<ADOP_MAX_LEVELS>, n, a.ncam, kPointWaves, 0, s, cams, a);
+  bool plain = a.radius == nullptr;
+  for (int k = 0; k < a.ncam; ++k) plain = plain && !cams.c[k].normals && camera_is_plain(cams.c[k]);
+#define ADOP_DEPTH(L)                                                                       \
+  return plain ? launch_strided(k_depth<L, true>, n, a.ncam, kPointWaves, 0, s, cams, a)    \
+               : launch_strided(k_depth<L, false>, n, a.ncam, kPointWaves, 0, s, cams, a)
+  switch (a.levels) {
+    case 1: ADOP_DEPTH(1);
+    case 2: ADOP_DEPTH(2);
+    case 3: ADOP_DEPTH(3);
+    case 4: ADOP_DEPTH(4);
+    case 5: ADOP_DEPTH(5);
+    default: ADOP_DEPTH(ADOP_MAX_LEVELS);
+  }
+#undef ADOP_DEPTH
 }
 
 cudaError_t launch_accum(const LaunchCams& cams, const PointArgs& a, int c, adop_dtype fd, cudaStream_t s) {
