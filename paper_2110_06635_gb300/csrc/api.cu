@@ -66,7 +66,7 @@ int prof_id(const char* name) {
 
 
 constexpr size_t kAlign = 256;
-constexpr int kMaxPartialBlocks = 4096;
+constexpr int kMaxPartialBlocks = 2048;  // (point_blocks: 8 per SM)
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
@@ -120,7 +120,7 @@ WsLayout layout(const adop_points* pts, const adop_camera* cams, int32_t n_cam, 
   L.bin_rows = bin_table_rows(n_cam);
   L.binning = true;
   L.partials = o;
-  o = align_up(o + (size_t)n_cam * kMaxPartialBlocks * 12 * 4);
+  o = align_up(o + (size_t)n_cam * kMaxPartialBlocks * 24 * 4);
   L.total = o;
   return L;
 }
@@ -455,7 +455,7 @@ WsLayout noalloc_layout(const adop_points* pts, const adop_camera* cams, int32_t
   }
   L.partials = o;
   const int chunk = n_cam < kMaxCamsPerLaunch ? n_cam : kMaxCamsPerLaunch;
-  o = align_up(o + (size_t)chunk * kMaxPartialBlocks * 12 * 4);
+  o = align_up(o + (size_t)chunk * kMaxPartialBlocks * 24 * 4);
   L.total = o;
   return L;
 }

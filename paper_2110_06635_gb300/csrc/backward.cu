@@ -232,23 +232,49 @@ __device__ __forceinline__ void write_point_grads(const BwdArgs& b, int64_t i, c
   }
 }
 
+// A sum as a pair of floats whose value is hi + lo, lo the rounding errors of
+// hi's additions (Knuth's TwoSum): the pose and intrinsics terms of a view
+// cancel, so that the rounding of plain FP32 sums over threads and blocks, in
+// whichever order the binning lists the points, reached 1e-6 of the result.
+struct Pair {
+  float hi, lo;
+};
+__device__ __forceinline__ Pair pair_add(Pair x, float y_hi, float y_lo) {
+  const float s = __fadd_rn(x.hi, y_hi);
+  const float t = __fsub_rn(s, x.hi);
+  const float err = __fadd_rn(__fsub_rn(x.hi, __fsub_rn(s, t)), __fsub_rn(y_hi, t));
+  return Pair{s, __fadd_rn(__fadd_rn(x.lo, y_lo), err)};
+}
+
+__device__ __forceinline__ Pair warp_sum(Pair v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    v = pair_add(v, __shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+  return v;
+}
+
+// A block's partial sum of term k (0 .. 11): [camera][hi of 12 terms, lo of 12][block].
+__device__ __forceinline__ void store_partial(const BwdArgs& b, int k, Pair v) {
+  float* at = b.partials + ((int64_t)blockIdx.y * 24 + k) * gridDim.x + blockIdx.x;
+  at[0] = v.hi;
+  at[12 * (int64_t)gridDim.x] = v.lo;
+}
+
 // Pose / intrinsics terms: warp shuffle -> shared memory -> one partial per block.
 __device__ __forceinline__ void block_partials(const BwdArgs& b, float (&red)[12]) {
-  __shared__ float sm[kThreads / 32][12];
+  __shared__ Pair sm[kThreads / 32][12];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
-    float v = red[k];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const Pair v = warp_sum(Pair{red[k], 0.0f});
     if (lane == 0) sm[warp][k] = v;
   }
   __syncthreads();
   if (threadIdx.x < 12) {
-    float v = 0.0f;
+    Pair v{0.0f, 0.0f};
 #pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) v += sm[w][threadIdx.x];
-    b.partials[((int64_t)blockIdx.y * 12 + threadIdx.x) * gridDim.x + blockIdx.x] = v;
+    for (int w = 0; w < kThreads / 32; ++w) v = pair_add(v, sm[w][threadIdx.x].hi, sm[w][threadIdx.x].lo);
+    store_partial(b, threadIdx.x, v);
   }
 }
 
@@ -635,11 +661,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_bwd_items(const __grid_constant
   if (b.partials != nullptr) {  // block sum of the pose / intrinsics terms: warp w takes terms w, w + 8
     __syncthreads();
     for (int k = warp; k < 12; k += kWarps) {
-      float t = 0.0f;
-      for (int j = lane; j < kThreads; j += 32) t += s_red[k][j];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0) b.partials[((int64_t)blockIdx.y * 12 + k) * gridDim.x + blockIdx.x] = t;
+      Pair t{0.0f, 0.0f};
+      for (int j = lane; j < kThreads; j += 32) t = pair_add(t, s_red[k][j], 0.0f);
+      t = warp_sum(t);
+      if (lane == 0) store_partial(b, k, t);
     }
   }
 }
@@ -802,7 +827,7 @@ __global__ void __launch_bounds__(kThreads) k_bin_scatter_blk(const __grid_const
 }
 
 // Block (k, camera) sums element k of the pose / intrinsics terms over all
-// block partials (laid out element-major, [camera][12][block], so that the
+// block partials (laid out element-major, [camera][24][block], so that the
 // loads coalesce): each thread a strided share, then the warps, then the
 // warp sums in order: a fixed order for given partials.
 constexpr int kReduceThreads = 256;
@@ -810,20 +835,21 @@ constexpr int kReduceThreads = 256;
 __global__ void __launch_bounds__(kReduceThreads) k_bwd_reduce(const float* __restrict__ partials, int blocks_x,
                                                                float* grad_pose, float* grad_intr) {
   pdl_entry();
-  __shared__ float sm[kReduceThreads / 32];
+  __shared__ Pair sm[kReduceThreads / 32];
   const int k = blockIdx.x, cam = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float* pk = partials + ((int64_t)cam * 12 + k) * blocks_x;
-  float v = 0.0f;
-  for (int bi = threadIdx.x; bi < blocks_x; bi += kReduceThreads) v += pk[bi];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const float* hi = partials + ((int64_t)cam * 24 + k) * blocks_x;
+  const float* lo = hi + 12 * (int64_t)blocks_x;
+  Pair v{0.0f, 0.0f};
+  for (int bi = threadIdx.x; bi < blocks_x; bi += kReduceThreads) v = pair_add(v, hi[bi], lo[bi]);
+  v = warp_sum(v);
   if (lane == 0) sm[warp] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
-    float t = 0.0f;
+    Pair r{0.0f, 0.0f};
 #pragma unroll
-    for (int w = 0; w < kReduceThreads / 32; ++w) t += sm[w];
+    for (int w = 0; w < kReduceThreads / 32; ++w) r = pair_add(r, sm[w].hi, sm[w].lo);
+    const float t = isfinite(r.hi) ? r.hi + r.lo : r.hi;
     if (k < 6) {
       if (grad_pose) grad_pose[cam * 6 + k] += t;
     } else if (grad_intr) {

@@ -88,7 +88,7 @@ enum GradMode : int32_t { kGradAssign = 0, kGradAccumulate = 1, kGradAtomic = 2 
 struct BwdArgs {
   float* grad_feat;
   float* grad_xyz;
-  float* partials;      // [ncam][12][blocks_x] pose (6) + intrinsics (6) block sums
+  float* partials;      // [ncam][24][blocks_x] pose (6) + intrinsics (6) block sums, their rounding errors
   int32_t mode;         // GradMode
   int32_t all_projected;
   int32_t feat_out;     // adop_dtype of grad_feat (16-bit types only with kGradAssign)
