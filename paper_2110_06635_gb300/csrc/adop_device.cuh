@@ -58,6 +58,7 @@ struct DevCam {
   int32_t* bin_list;         // visible point indices, tile by tile (NULL: no binning)
   int32_t* bin_table;        // [block][tile]: a binning block's first slot within the tile's range
   int32_t bin_rows;          // binning blocks the table has rows for
+  uint32_t* bin_bits;        // a bit per point: in some Lambda (whole 16 bytes)
   // photometric epilogue (Sec. 3.3); ev_scale = 2^-EV, computed on the host
   int32_t epi;
   int32_t leaky;  // training response curve (Eq. resonseleak) instead of clamping

@@ -74,13 +74,14 @@ bool finite(float v) { return std::isfinite(v); }
 
 // Workspace: per camera [keys | counts | sums | point layer masks | backward
 // pixel info | pixel-major upstream gradient | tile counts | tile offsets |
-// tile-ordered point list | the depth pass's per-point layer bytes], then the
+// tile-ordered point list | the depth pass's per-point layer bytes | a bit per
+// point, in some Lambda or not | binning blocks' first slots], then the
 // pose/intrinsics block partials.
 struct WsLayout {
   size_t key[ADOP_MAX_CAMERAS], cnt[ADOP_MAX_CAMERAS], acc[ADOP_MAX_CAMERAS], vis[ADOP_MAX_CAMERAS];
   size_t info[ADOP_MAX_CAMERAS], gpm[ADOP_MAX_CAMERAS];
   size_t bin_count[ADOP_MAX_CAMERAS], bin_off[ADOP_MAX_CAMERAS], bin_list[ADOP_MAX_CAMERAS];
-  size_t early[ADOP_MAX_CAMERAS], bin_table[ADOP_MAX_CAMERAS];
+  size_t early[ADOP_MAX_CAMERAS], bin_table[ADOP_MAX_CAMERAS], bin_bits[ADOP_MAX_CAMERAS];
   int32_t bin_rows;
   bool binning;
   size_t partials;
@@ -114,6 +115,8 @@ WsLayout layout(const adop_points* pts, const adop_camera* cams, int32_t n_cam, 
     o = align_up(o + (size_t)pts->n * 4);
     L.early[k] = o;
     o = align_up(o + (size_t)pts->n);
+    L.bin_bits[k] = o;
+    o = align_up(o + ((size_t)pts->n + 127) / 128 * 16);
     L.bin_table[k] = o;
     if (tiles <= (size_t)kBinSmemTiles) o = align_up(o + (size_t)bin_table_rows(n_cam) * tiles * 4);
   }
@@ -265,6 +268,7 @@ void fill_cam(DevCam& d, const adop_camera& cam, const adop_frame* f, bool use_f
     d.bin_list = reinterpret_cast<int32_t*>(ws + L.bin_list[k]);
     d.bin_table = reinterpret_cast<int32_t*>(ws + L.bin_table[k]);
     d.bin_rows = L.bin_rows;
+    d.bin_bits = reinterpret_cast<uint32_t*>(ws + L.bin_bits[k]);
   }
 }
 
@@ -603,10 +607,6 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
       }
     }
     const PointArgs a = point_args(pts, params, nc);
-    if ((e = timed("bwd_prepass", s, [&] { return launch_bwd_prepass(lc, a, pts->c, s); })) != cudaSuccess)
-      return cuda_fail(e, "backward prepass launch");
-    if (pts->n == 0) continue;
-    const int bx = point_blocks(pts->n, nc) < kMaxPartialBlocks ? point_blocks(pts->n, nc) : kMaxPartialBlocks;
     BwdArgs b{};
     b.grad_feat = grad_feat;
     b.grad_xyz = grad_xyz;
@@ -616,20 +616,37 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
     b.feat_out = params->grad_feat_dtype;
     bool dense = !b.all_projected;
     for (int j = 0; j < nc; ++j) dense = dense && lc.c[j].vis != nullptr;
-    if (dense) {
-      if ((e = timed("bwd_bin", s, [&] { return launch_bin(lc, a, b, pts->c, s); })) != cudaSuccess)
-        return cuda_fail(e, "backward binning launch");
-    } else {
+    if (!dense)
       for (int j = 0; j < nc; ++j) lc.c[j].bin_list = nullptr;
+    if (dense && pts->n > 0 &&
+        (e = timed("bwd_bin", s, [&] { return launch_bin(lc, a, b, pts->c, s); })) != cudaSuccess)
+      return cuda_fail(e, "backward binning launch");
+    // the prepass and the point pass that reads its records, a few cameras at a time
+    const int per = cams_per_backward(pts->n, nc);
+    for (int j0 = 0; j0 < nc; j0 += per) {
+      const int m = nc - j0 < per ? nc - j0 : per;
+      LaunchCams part;
+      const LaunchCams* lp = &lc;
+      if (m < nc) {
+        for (int j = 0; j < m; ++j) part.c[j] = lc.c[j0 + j];
+        lp = &part;
+      }
+      PointArgs pa = a;
+      pa.ncam = m;
+      if ((e = timed("bwd_prepass", s, [&] { return launch_bwd_prepass(*lp, pa, pts->c, s); })) != cudaSuccess)
+        return cuda_fail(e, "backward prepass launch");
+      if (pts->n == 0) continue;
+      const int bx = point_blocks(pts->n, m) < kMaxPartialBlocks ? point_blocks(pts->n, m) : kMaxPartialBlocks;
+      if ((e = timed("bwd_points", s, [&] {
+             return launch_bwd_points(*lp, pa, b, pts->c, pts->feat_dtype, bx, s);
+           })) != cudaSuccess)
+        return cuda_fail(e, "backward point pass launch");
+      if (want_pose && (e = timed("bwd_reduce", s, [&] {
+                          return launch_bwd_reduce(b.partials, m, bx, grad_pose ? grad_pose + 6 * (k0 + j0) : nullptr,
+                                                   grad_intr ? grad_intr + 6 * (k0 + j0) : nullptr, s);
+                        })) != cudaSuccess)
+        return cuda_fail(e, "backward reduce launch");
     }
-    if ((e = timed("bwd_points", s, [&] { return launch_bwd_points(lc, a, b, pts->c, pts->feat_dtype, bx, s); })) !=
-        cudaSuccess)
-      return cuda_fail(e, "backward point pass launch");
-    if (want_pose && (e = timed("bwd_reduce", s, [&] {
-                        return launch_bwd_reduce(b.partials, nc, bx, grad_pose ? grad_pose + 6 * k0 : nullptr,
-                                                 grad_intr ? grad_intr + 6 * k0 : nullptr, s);
-                      })) != cudaSuccess)
-      return cuda_fail(e, "backward reduce launch");
   }
   g_last_error.clear();
   return ADOP_OK;

@@ -232,6 +232,29 @@ __device__ __forceinline__ void write_point_grads(const BwdArgs& b, int64_t i, c
   }
 }
 
+// Zero gradients of the 32 points from i0 (a multiple of 32), by a warp: whole
+// rows of 32 C elements and 96 floats, as 16-byte streaming stores.
+template <int C>
+__device__ __forceinline__ void zero_chunk(const BwdArgs& b, int64_t i0, int lane, bool xyz16) {
+  const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (b.grad_feat) {  // 16-byte aligned; 32 C values are a multiple of 16 bytes in every type
+    const int size = b.feat_out == ADOP_F32 ? 4 : 2;
+    float4* dst = reinterpret_cast<float4*>(reinterpret_cast<char*>(b.grad_feat) + i0 * (C * size));
+#pragma unroll
+    for (int v = 0; v < (32 * C * 4 / 16 + 31) / 32; ++v)
+      if (v * 32 + lane < 32 * C * size / 16) __stcs(dst + v * 32 + lane, z);
+  }
+  if (b.grad_xyz) {
+    float* dst = b.grad_xyz + 3 * i0;
+    if (xyz16) {
+      if (lane < 24) __stcs(reinterpret_cast<float4*>(dst) + lane, z);
+    } else {
+#pragma unroll
+      for (int v = 0; v < 3; ++v) __stcs(dst + v * 32 + lane, 0.0f);
+    }
+  }
+}
+
 // A sum as a pair of floats whose value is hi + lo, lo the rounding errors of
 // hi's additions (Knuth's TwoSum): the pose and intrinsics terms of a view
 // cancel, so that the rounding of plain FP32 sums over threads and blocks, in
@@ -641,21 +664,34 @@ __global__ void __launch_bounds__(kThreads, 4) k_bwd_items(const __grid_constant
   if (BINNED && b.mode == kGradAssign) {
     // the points in no Lambda get zero gradients here: streaming stores that
     // overlap the blocks still busy with latency-bound pairs (in the binning
-    // kernel they cost 34 us, here 24).  Four grid-stride steps at a time, so
-    // that their mask loads are in flight together while each store still
-    // covers consecutive points across the warp (point pass 170 -> 166 us on
-    // the 5M-point view, 959 -> 890 us on the 120M-point frame; two at a time
-    // 167 / 870 us)
-    const float zf[C] = {};
-    const float zx[3] = {0.0f, 0.0f, 0.0f};
-    const int64_t S = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < a.n; i0 += 4 * S) {
-      uint32_t m[4];
+    // kernel they cost 34 us, here 24).  The binning's bit per point says which
+    // they are: a warp takes 128 points, whose 16 bytes of bits it reads one
+    // step ahead, and writes each 32 points that are all zero with 16-byte
+    // stores.  (Reading the 4-byte masks again and storing 12 bytes per lane,
+    // the whole pass took 887 us on the 120M-point frame, 807 now.)
+    const int64_t words = (a.n + 31) / 32;
+    const int64_t S = (int64_t)gridDim.x * kWarps * 4;
+    const bool xyz16 = ((uintptr_t)b.grad_xyz & 15u) == 0u;
+    auto bits_at = [&](int64_t w0) -> uint4 {  // (the array is padded to whole uint4s)
+      return w0 < words ? __ldcs(reinterpret_cast<const uint4*>(cam.bin_bits + w0)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    int64_t w0 = ((int64_t)blockIdx.x * kWarps + warp) * 4;
+    uint4 ahead = bits_at(w0);
+    for (; w0 < words; w0 += S) {
+      const uint32_t m[4] = {ahead.x, ahead.y, ahead.z, ahead.w};
+      ahead = bits_at(w0 + S);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) m[u] = i0 + u * S < a.n ? (__ldcs(cam.vis + i0 + u * S) & 0xFFu) : 1u;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (m[u] == 0u) write_point_grads<C>(b, i0 + u * S, zf, zx, false);
+      for (int u = 0; u < 4; ++u) {
+        const int64_t i0 = (w0 + u) * 32;
+        if (i0 >= a.n) break;
+        if (m[u] == 0u && i0 + 32 <= a.n) {
+          zero_chunk<C>(b, i0, lane, xyz16);
+        } else if (i0 + lane < a.n && !((m[u] >> lane) & 1u)) {
+          const float zf[C] = {};
+          const float zx[3] = {0.0f, 0.0f, 0.0f};
+          write_point_grads<C>(b, i0 + lane, zf, zx, false);
+        }
+      }
     }
   }
   if (b.partials != nullptr) {  // block sum of the pose / intrinsics terms: warp w takes terms w, w + 8
@@ -696,6 +732,8 @@ __global__ void __launch_bounds__(kThreads) k_bin_count(const __grid_constant__ 
     const int64_t i = base + lane;
     const uint32_t v = i < a.n ? __ldg(cam.vis + i) : 0u;
     const bool active = (v & 0xFFu) != 0u;
+    const unsigned bits = __ballot_sync(0xffffffffu, active);
+    if (lane == 0) cam.bin_bits[base >> 5] = bits;
     const uint32_t tile = min(v >> 8, (uint32_t)cam.tiles - 1u);
     int head, len, rank;
     lane_run(tile, active, lane, head, len, rank);
@@ -778,26 +816,62 @@ __global__ void __launch_bounds__(kThreads) k_bin_scatter(const __grid_constant_
 // 120M-point frame 267 -> 194 us; unchanged on the 5M-point view).
 constexpr int kBinBlocksPerSm = 8;
 
+// (whole 128 points per block: a warp reads 4 masks a lane)
 __device__ __forceinline__ void chunk_of(int64_t n, int64_t& c0, int64_t& c1) {
-  const int64_t per = (n + gridDim.x - 1) / gridDim.x;
-  c0 = (int64_t)blockIdx.x * per;
+  const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 127) / 128 * 128;
+  c0 = min(n, (int64_t)blockIdx.x * per);
   c1 = min(n, c0 + per);
 }
 
+constexpr int kBinStep = kThreads / 32 * 128;  // points of a block's step: 128 a warp
+constexpr int kBinAhead = 2;                   // steps whose loads are in flight together
+
+// The count also writes a bit per point (in some Lambda or not), which the
+// scatter and the zero-gradient tail read instead of the masks: 15 MB instead
+// of 480 for 120M points (count, scan and scatter 200 -> 173 us).  Bound by the
+// mask stream: 16 bytes a lane and step where the masks are 16-byte aligned.
 __global__ void __launch_bounds__(kThreads) k_bin_count_blk(const __grid_constant__ LaunchCams cams,
                                                             const __grid_constant__ PointArgs a) {
   pdl_entry();
   extern __shared__ int32_t bins[];
   const DevCam& cam = cams.c[blockIdx.y];
   const int T = cam.tiles;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool vis16 = ((uintptr_t)cam.vis & 15u) == 0u;
   for (int t = threadIdx.x; t < T; t += blockDim.x) bins[t] = 0;
   __syncthreads();
   int64_t c0, c1;
   chunk_of(a.n, c0, c1);
-#pragma unroll 4
-  for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-    const uint32_t v = __ldg(cam.vis + i);
-    if (v & 0xFFu) atomicAdd(bins + min(v >> 8, (uint32_t)T - 1u), 1);
+  for (int64_t base = c0 + warp * 128; base < c1; base += kBinAhead * kBinStep) {
+    uint32_t v[kBinAhead][4];
+#pragma unroll
+    for (int s = 0; s < kBinAhead; ++s) {
+      const int64_t i = base + s * kBinStep + lane * 4;
+      if (vis16 && i + 4 <= c1) {
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(cam.vis + i));
+        v[s][0] = q.x; v[s][1] = q.y; v[s][2] = q.z; v[s][3] = q.w;
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[s][u] = i + u < c1 ? __ldg(cam.vis + i + u) : 0u;
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < kBinAhead; ++s) {
+      const int64_t at = base + s * kBinStep;
+      if (at >= c1) break;
+      uint32_t bits = 0u;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v[s][u] & 0xFFu) {
+          bits |= 1u << u;
+          atomicAdd(bins + min(v[s][u] >> 8, (uint32_t)T - 1u), 1);
+        }
+      // 8 lanes' 4 bits make a word
+      bits <<= 4 * (lane & 7);
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) bits |= __shfl_xor_sync(0xffffffffu, bits, o);
+      if ((lane & 7) == 0 && at + lane * 4 < c1) cam.bin_bits[(at >> 5) + (lane >> 3)] = bits;
+    }
   }
   __syncthreads();
   int32_t* row = cam.bin_table + (int64_t)blockIdx.x * T;
@@ -815,14 +889,38 @@ __global__ void __launch_bounds__(kThreads) k_bin_scatter_blk(const __grid_const
   extern __shared__ int32_t bins[];  // this block's next slot per tile
   const DevCam& cam = cams.c[blockIdx.y];
   const int T = cam.tiles;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t* row = cam.bin_table + (int64_t)blockIdx.x * T;
   for (int t = threadIdx.x; t < T; t += blockDim.x) bins[t] = cam.bin_off[t] + row[t];
   __syncthreads();
   int64_t c0, c1;
   chunk_of(a.n, c0, c1);
-  for (int64_t i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
-    const uint32_t v = __ldg(cam.vis + i);
-    if (v & 0xFFu) cam.bin_list[atomicAdd(bins + min(v >> 8, (uint32_t)T - 1u), 1)] = (int32_t)i;
+  // two steps' bits at once; then 32 consecutive points a load, so that
+  // neighbours take neighbouring slots (four consecutive points a lane
+  // instead: the point pass of 12 views of 20M points took 1851 us, not 1740)
+  constexpr int kWords = 2;
+  for (int64_t base = c0 + warp * 128; base < c1; base += kWords * kBinStep) {
+    uint32_t bits[kWords][4];
+#pragma unroll
+    for (int s = 0; s < kWords; ++s) {
+      const int64_t at = base + s * kBinStep;  // (a multiple of 128: whole 16 bytes of bits)
+      const uint4 q = at < c1 ? __ldg(reinterpret_cast<const uint4*>(cam.bin_bits + (at >> 5))) : make_uint4(0u, 0u, 0u, 0u);
+      bits[s][0] = q.x; bits[s][1] = q.y; bits[s][2] = q.z; bits[s][3] = q.w;
+    }
+#pragma unroll
+    for (int s = 0; s < kWords; ++s) {
+      if ((bits[s][0] | bits[s][1] | bits[s][2] | bits[s][3]) == 0u) continue;
+      uint32_t v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int64_t i = base + s * kBinStep + u * 32 + lane;
+        v[u] = i < c1 && ((bits[s][u] >> lane) & 1u) ? __ldg(cam.vis + i) : 0u;  // (bits past c1 were never written)
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v[u] & 0xFFu)
+          cam.bin_list[atomicAdd(bins + min(v[u] >> 8, (uint32_t)T - 1u), 1)] = (int32_t)(base + s * kBinStep + u * 32 + lane);
+    }
   }
 }
 

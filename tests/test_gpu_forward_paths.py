@@ -27,7 +27,8 @@ def _camera(w, h, **kw):
     (312_001, 8, "f32", 4, 2200, 1500, False),
     (40_001, 16, "f16", 3, 1400, 1000, True),
     (40_001, 3, "f32", 5, 2400, 2001, True),
-    (20_011, 1, "f32", 8, 3000, 2400, False)])
+    (20_011, 1, "f32", 8, 3000, 2400, False),
+    (20_011, 2, "f32", 2, 4128, 2080, True)])   # more screen tiles than the binning counts per block
 def test_forward_and_backward_paths(adop, orc, n, c, dtype, levels, w, h, keep):
     sc = scenes.tiny_spheres(n, c, seed=n % 1000)
     cams = [_camera(w, h)]
@@ -39,6 +40,39 @@ def test_forward_and_backward_paths(adop, orc, n, c, dtype, levels, w, h, keep):
         fr = g["frames"][0]
         acc = fr.acc.view(-1, c).cpu().numpy()
         assert not acc[r["cnt"][0] == 0].any()
+
+
+@pytest.mark.parametrize("keep", [True, False])
+def test_several_cameras_of_a_large_cloud(adop, keep):
+    """From 4M points on the backward takes the cameras two at a time: the
+    same gradients as one call per camera, summed, and the same pose rows
+    (FP32 sums in another order)."""
+    import torch
+    from parity import assert_close
+    n = (1 << 22) + 3
+    sc = scenes.tiny_spheres(n, 4, seed=9)
+    cams = [_camera(200 + 16 * k, 150) for k in range(3)]
+    pts = adop.Points(torch.from_numpy(sc.xyz).cuda(), torch.from_numpy(sc.feat).cuda())
+    params = adop.Params(4, 0.01, 1e-3, None, adop.ADOP_FLAG_GRAD_ASSIGN)
+    G = [[torch.from_numpy(g).cuda() for g in scenes.upstream_grad(c.w, c.h, 4, 4, 30 + k)]
+         for k, c in enumerate(cams)]
+
+    def grads(sub, g):
+        frames = [adop.Frame.alloc(c, 4, 4, torch.float32, keep, "cuda", n if keep else None) for c in sub]
+        ws = adop.alloc_workspace(pts, sub, params)
+        adop.adop_render_forward(pts, sub, params, frames, ws)
+        out = [torch.full((n, 4), float("nan"), device="cuda"), torch.full((n, 3), float("nan"), device="cuda"),
+               torch.zeros((len(sub), 6), device="cuda"), torch.zeros((len(sub), 6), device="cuda")]
+        adop.adop_render_backward(pts, sub, params, frames, g, *out, ws)
+        return [o.cpu().numpy().astype(np.float64) for o in out]
+
+    got = grads(cams, G)
+    one = [grads([c], [g]) for c, g in zip(cams, G)]
+    for j in range(2):
+        assert_close(got[j], sum(o[j] for o in one), 1e-5, "per-point gradients")
+    for j in (2, 3):
+        want = np.concatenate([o[j] for o in one])
+        assert np.all(np.abs(got[j] - want) <= 1e-4 * np.abs(want).max())
 
 
 def test_layer_masks_only_4_byte_aligned(adop):
