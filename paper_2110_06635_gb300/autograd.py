@@ -49,8 +49,15 @@ def apply_tangent(cam, xi):
 
 def _effective_cameras(cameras, xi, intrinsics):
     cams = []
-    xi_h = None if xi is None else xi.detach().to("cpu", torch.float64).numpy()
-    k_h = None if intrinsics is None else intrinsics.detach().to("cpu", torch.float64).numpy()
+    if xi is not None and intrinsics is not None and xi.is_cuda and xi.device == intrinsics.device and \
+            xi.dtype == intrinsics.dtype == torch.float32:
+        # one copy to the host, so one wait for the GPU, instead of two
+        both = torch.cat([xi.detach().reshape(-1), intrinsics.detach().reshape(-1)]).cpu().numpy().astype(np.float64)
+        xi_h = both[:xi.numel()].reshape(xi.shape)
+        k_h = both[xi.numel():].reshape(intrinsics.shape)
+    else:
+        xi_h = None if xi is None else xi.detach().to("cpu", torch.float64).numpy()
+        k_h = None if intrinsics is None else intrinsics.detach().to("cpu", torch.float64).numpy()
     for k, cam in enumerate(cameras):
         c = apply_tangent(cam, xi_h[k]) if xi_h is not None and np.any(xi_h[k] != 0) else copy.copy(cam)
         if k_h is not None:
