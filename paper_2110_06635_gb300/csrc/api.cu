@@ -616,9 +616,10 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
     b.feat_out = params->grad_feat_dtype;
     bool dense = !b.all_projected;
     for (int j = 0; j < nc; ++j) dense = dense && lc.c[j].vis != nullptr;
-    if (!dense)
+    const bool bin = dense && pts->n > 0 && binning_pays(lc, a);
+    if (!bin)
       for (int j = 0; j < nc; ++j) lc.c[j].bin_list = nullptr;
-    if (dense && pts->n > 0 &&
+    if (bin &&
         (e = timed("bwd_bin", s, [&] { return launch_bin(lc, a, b, pts->c, s); })) != cudaSuccess)
       return cuda_fail(e, "backward binning launch");
     // the prepass and the point pass that reads its records, a few cameras at a time

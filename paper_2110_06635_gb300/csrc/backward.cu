@@ -988,6 +988,22 @@ cudaError_t launch_bwd_points(const LaunchCams& cams, const PointArgs& a, const 
   return e;
 }
 
+// Below 800 thousand points the four binning launches cost more than the
+// locality of the point pass gains, and so they do with fewer than some 500
+// points per tile, where a tile's points hardly share pixel records (step as
+// a CUDA graph, us, binned / in index order, BF16):
+//   20 thousand points, 640x400, surface 60.5 / 48.5, random 65.6 / 46.3
+//   600 thousand, 640x400, surface 88.1 / 80.3, random 116 / 93; 1080p, surface 217 / 221
+//   1.2M, 1080p (590 a tile), surface 269 / 280, random 242 / 200
+//   2.5M, 1080p, surface 317 / 373, random 408 / 400
+//   5M, 640x400, random 247 / 313
+//   1M, 3000x2400 (142 a tile), random 671 / 442
+bool binning_pays(const LaunchCams& cams, const PointArgs& a) {
+  int most = 0;
+  for (int k = 0; k < a.ncam; ++k) most = cams.c[k].tiles > most ? cams.c[k].tiles : most;
+  return a.n * a.ncam >= 800000 && a.n >= 500 * (int64_t)most;
+}
+
 cudaError_t launch_bin(const LaunchCams& cams, const PointArgs& a, const BwdArgs& b, int c, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   for (int k = 0; k < a.ncam; ++k) {
@@ -999,6 +1015,10 @@ cudaError_t launch_bin(const LaunchCams& cams, const PointArgs& a, const BwdArgs
   if (most <= kBinSmemTiles) {
     const size_t smem = sizeof(int32_t) * (size_t)most;
     int64_t want = (int64_t)num_sms() * kBinBlocksPerSm;
+    // a block clears and writes a row of all tiles: with fewer than two points
+    // per tile and block, fewer blocks, down to one per SM
+    const int64_t rows = a.n / (2 * (int64_t)most);
+    if (rows * a.ncam < want) want = rows * a.ncam > num_sms() ? rows * a.ncam : num_sms();
     want = (want + a.ncam - 1) / a.ncam;
     for (int k = 0; k < a.ncam; ++k) want = want < cams.c[k].bin_rows ? want : cams.c[k].bin_rows;
     const dim3 grid((unsigned)(want < 1 ? 1 : want), a.ncam);

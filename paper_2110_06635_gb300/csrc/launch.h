@@ -150,6 +150,8 @@ cudaError_t launch_bwd_points(const LaunchCams& cams, const PointArgs& a, const 
 // Screen-tile binning of the visible points (backward): count, scan, scatter.
 // (The binned point pass then also writes the zero gradients of the points
 // that are in no Lambda when the mode is kGradAssign.)
+// (bits, list and tile offsets; launched where binning_pays.)
+bool binning_pays(const LaunchCams& cams, const PointArgs& a);
 cudaError_t launch_bin(const LaunchCams& cams, const PointArgs& a, const BwdArgs& b, int c, cudaStream_t s);
 cudaError_t launch_bwd_reduce(const float* partials, int ncam, int blocks_x, float* grad_pose,
                               float* grad_intr, cudaStream_t s);
