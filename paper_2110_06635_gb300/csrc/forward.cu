@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kThreads) k_seed(const __grid_constant__ Launc
 // tests is written for the backward pass, with the point's layer-0 screen
 // tile in bits 8..31 (where the caller or a backward reads it: cam.vis).
 //
-// A warp takes 32 kPerLane consecutive points, reads the depth pass's layer
+// A warp takes 32, 64 or 128 consecutive points, reads the depth pass's layer
 // bytes (cam.early) and lists the points with a layer left; those are then
 // projected again and tested, one per lane, so that the points which the
 // depth pass ruled out -- outside the view, or hidden when they were met --
@@ -276,12 +276,14 @@ __global__ void __launch_bounds__(kAccumThreads, accum_min_blocks<C, kL>())
     if (i >= cam.n) return 0u;
     if (!early) {
       const int64_t left = cam.n - i;
-      return per_lane == 1 ? 0xFFu : (left >= 4 ? ~0u : ~0u >> (8 * (4 - (int)left)));
+      return ~0u >> (8 * (4 - (int)(left < per_lane ? left : per_lane)));
     }
     if (per_lane == 1) return (uint32_t)__ldcs(cam.early + i);
-    if (i + kPerLane <= cam.n) return __ldcs(reinterpret_cast<const uint32_t*>(cam.early + i));
+    if (i + per_lane <= cam.n)
+      return per_lane == 2 ? (uint32_t)__ldcs(reinterpret_cast<const uint16_t*>(cam.early + i))
+                           : __ldcs(reinterpret_cast<const uint32_t*>(cam.early + i));
     uint32_t w = 0u;
-    for (int u = 0; u < kPerLane && i + u < cam.n; ++u) w |= (uint32_t)__ldcs(cam.early + i + u) << (8 * u);
+    for (int u = 0; u < per_lane && i + u < cam.n; ++u) w |= (uint32_t)__ldcs(cam.early + i + u) << (8 * u);
     return w;
   };
   int64_t base = ((int64_t)blockIdx.x * (kAccumThreads / 32) + warp) * 32 * per_lane;
@@ -455,6 +457,8 @@ cudaError_t launch_seed(const LaunchCams& cams, const PointArgs& a, int c, adop_
 //   C = 8, 121 MB, 2.6M points:  106 without,  101 with
 //   C = 8, 121 MB, 5M points:    116 without,  111 with
 //   C = 4, 308 MB, 120M points:  808 without,  573 with
+// (Requiring a point per two pixels as well made the 1080p step of 1.2M points
+// slower, 270 -> 277 us.)
 int seed_rule(const LaunchCams& cams, const PointArgs& a, int c) {
   int64_t px = 0;
   for (int k = 0; k < a.ncam; ++k) px += cams.c[k].off[a.levels];
@@ -489,9 +493,12 @@ cudaError_t launch_depth(const LaunchCams& cams, const PointArgs& a, cudaStream_
 cudaError_t launch_accum(const LaunchCams& cams, const PointArgs& a, int c, adop_dtype fd, cudaStream_t s) {
   const int64_t n = most_points(cams, a);
   if (n == 0) return cudaSuccess;
-  // one point a lane where four would leave SMs without work (20 thousand
-  // points: 9.0 us, 15.3 with four; 778 thousand: 27 us, 24 with four)
-  const int per_lane = n * a.ncam >= (int64_t)num_sms() * 16 * 32 * kPerLane ? kPerLane : 1;
+  // four points a lane where that leaves 2.5 waves of resident warps, else two
+  // or one, which skip less but fill the last wave (C = 4 at 1080p, us with
+  // 1 / 2 / 4 a lane: 400 thousand points 19.0 / 20.7 / 21.6, 1.2M 28.9 / 29.5 /
+  // 32.9, 3.5M 52.5 / 50.0 / 49.9, 8M 92.8 / 82.0 / 77.9, in random order 127 / 96 / 87)
+  int per_lane = kPerLane;
+  while (per_lane > 1 && 2 * n * a.ncam < 5 * (int64_t)num_sms() * 48 * 32 * per_lane) per_lane /= 2;
   const int64_t work = (n + per_lane - 1) / per_lane;
   cudaError_t e = cudaSuccess;
 #define ADOP_ACCUM(L)                                                                                       \

@@ -1,6 +1,6 @@
 """The forward's launch-time choices against the oracle: sums seeded with each
-pixel's nearest point (from 96 MB of pixel state) or cleared, one or four
-points a lane in the accumulate pass (from 311296 points on 152 SMs), every
+pixel's nearest point (from 96 MB of pixel state) or cleared, one, two
+or four points a lane in the accumulate pass (from 1167360 and 2334720 points on 152 SMs), every
 depth-pass layer count, state kept or rendered again by the backward, and a
 layer-mask buffer that is only 4-byte aligned."""
 import numpy as np
@@ -18,17 +18,21 @@ def _camera(w, h, **kw):
 
 
 @pytest.mark.parametrize("n,c,dtype,levels,w,h,keep", [
-    (311_295, 4, "f32", 4, 320, 200, True),     # one point a lane
-    (311_297, 4, "f32", 4, 320, 200, True),     # four, and a last chunk of one point
+    (1_167_359, 4, "f32", 4, 320, 200, True),   # one point a lane
+    (1_167_361, 4, "f32", 4, 320, 200, True),   # two, and a last chunk of one point
+    (2_334_721, 4, "f32", 4, 320, 200, False),  # four, and a last chunk of one point
     (400_003, 8, "bf16", 5, 333, 217, False),
     (350_001, 2, "f16", 2, 320, 200, True),
     (350_001, 1, "f32", 1, 320, 200, False),
     (40_001, 8, "bf16", 4, 2200, 1500, True),   # seeded
-    (312_001, 8, "f32", 4, 2200, 1500, False),
+    (2_200_001, 8, "f32", 4, 2200, 1500, False),
     (40_001, 16, "f16", 3, 1400, 1000, True),
     (40_001, 3, "f32", 5, 2400, 2001, True),
     (20_011, 1, "f32", 8, 3000, 2400, False),
-    (20_011, 2, "f32", 2, 4128, 2080, True)])   # more screen tiles than the binning counts per block
+    (799_999, 4, "bf16", 4, 320, 200, True),    # backward in index order, and binned from 800000 on
+    (800_003, 4, "bf16", 4, 320, 200, True),
+    (800_003, 8, "f32", 4, 1600, 1100, False),  # in index order: fewer than 500 points a tile
+    (4_200_003, 2, "f32", 2, 4128, 2080, True)])   # binned, more tiles than a block counts in shared memory
 def test_forward_and_backward_paths(adop, orc, n, c, dtype, levels, w, h, keep):
     sc = scenes.tiny_spheres(n, c, seed=n % 1000)
     cams = [_camera(w, h)]
@@ -75,9 +79,40 @@ def test_several_cameras_of_a_large_cloud(adop, keep):
         assert np.all(np.abs(got[j] - want) <= 1e-4 * np.abs(want).max())
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_binned_gradient_buffers_only_aligned_as_asked(adop, dtype):
+    """dL/dx 4 bytes past a 16-byte boundary, and dL/dtau in 16 bits, give the
+    zero gradients and the others of an aligned call (binned, a point count
+    that is no multiple of 32, buffers filled with NaN).  A point's sum over
+    its layers is split where the list of a warp's pairs is, so that FP32
+    rounding may differ, and with it one step of FP16."""
+    import torch
+    from parity import assert_close
+    n, c = 800_021, 3
+    sc = scenes.tiny_spheres(n, c, seed=3)
+    cam = _camera(320, 200)
+    pts = adop.Points(torch.from_numpy(sc.xyz).cuda(), torch.from_numpy(sc.feat).cuda())
+    params = adop.Params(4, 0.01, 1e-3, None, adop.ADOP_FLAG_GRAD_ASSIGN)
+    fr = adop.Frame.alloc(cam, c, 4, torch.float32, True, "cuda", n)
+    ws = adop.alloc_workspace(pts, [cam], params)
+    adop.adop_render_forward(pts, [cam], params, [fr], ws)
+    G = [[torch.from_numpy(g).cuda() for g in scenes.upstream_grad(cam.w, cam.h, 4, c, 8)]]
+    got = []
+    for offset in (0, 1):
+        gx = torch.full((n * 3 + 4,), float("nan"), device="cuda")[offset:offset + n * 3].view(n, 3)
+        assert gx.data_ptr() % 16 == 4 * offset
+        gf = torch.full((n, c), float("nan"), dtype=torch.float16 if dtype == "f16" else torch.float32, device="cuda")
+        adop.adop_render_backward(pts, [cam], params, [fr], G, gf, gx, None, None, ws)
+        got.append((gf.float().cpu().numpy(), gx.cpu().numpy()))
+    assert_close(got[0][0], got[1][0], 1e-6 if dtype == "f32" else 2e-3, "dL/dtau")
+    assert_close(got[0][1], got[1][1], 1e-5, "dL/dx")
+    unseen = fr.vis.cpu().numpy() & 0xFF == 0
+    assert unseen.any() and not got[0][0][unseen].any() and not got[0][1][unseen].any()
+
+
 def test_layer_masks_only_4_byte_aligned(adop):
     import torch
-    sc = scenes.tiny_spheres(311_303, 4, seed=5)
+    sc = scenes.tiny_spheres(2_334_731, 4, seed=5)
     cam = _camera(320, 200)
     pts = adop.Points(torch.from_numpy(sc.xyz).cuda(), torch.from_numpy(sc.feat).cuda())
     params = adop.Params(4, 0.01, 1e-3, None, 0)
