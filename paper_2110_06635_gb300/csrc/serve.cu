@@ -156,10 +156,11 @@ void Server::admit_locked() {
     if (off == SIZE_MAX) break;  // strict FIFO: the head waits for memory
     r.offset = off;
     // a byte per point lets the accumulate pass skip what the depth pass ruled
-    // out (sixteen requests over 8M points: 3.08 -> 2.71 ms); taken while less than half of the pool is in use, so
-    // that a full pool holds pixel state
+    // out (sixteen requests over 8M points: 3.08 -> 2.71 ms); taken where the
+    // pool would hold eight such requests, so that it costs no concurrency
+    // where the pool is small
     const size_t n = (size_t)clouds[r.cloud].n;
-    if (alloc.in_use() + alloc.round(n) <= alloc.capacity() / 2) r.early = alloc.alloc(n);
+    if (8 * (alloc.round(r.bytes) + alloc.round(n)) <= alloc.capacity()) r.early = alloc.alloc(n);
     r.state = kAdmitted;
     admitted.push_back(r.ticket);
     queue.pop();
