@@ -310,7 +310,7 @@ def recorded_atomics(kernel: str):
 
 
 # bench name of each library kernel (the k_bin_* launches are one entry)
-NCU_KERNELS = {"k_clear": "clear", "k_depth": "depth", "k_accum": "accumulate", "k_normalize": "normalize",
+NCU_KERNELS = {"k_clear": "clear", "k_depth": "depth", "k_seed": "seed", "k_accum": "accumulate", "k_normalize": "normalize",
                "k_bwd_prepass": "bwd_prepass", "k_bin_count_blk": "bwd_bin", "k_bin_scan": "bwd_bin",
                "k_bin_scatter_blk": "bwd_bin", "k_bwd_items": "bwd_points", "k_bwd_reduce": "bwd_reduce"}
 NCU_SOURCES = {"forward": ["paper_2110_06635_gb300/csrc/forward.cu", "paper_2110_06635_gb300/csrc/adop_device.cuh"],
@@ -357,7 +357,7 @@ def record_traffic(csv_paths) -> dict:
         dur = sum(np.mean([x.get("gpu__time_duration.sum", 0) for x in v]) for v in per_kernel.values())
         busy = max(np.mean([x.get("lts__d_atomic_input_cycles_active.avg.pct_of_peak_sustained_elapsed", 0)
                             for x in v]) for v in per_kernel.values())
-        src = NCU_SOURCES["forward" if name in ("clear", "depth", "accumulate", "normalize") else "backward"]
+        src = NCU_SOURCES["forward" if name in ("clear", "depth", "seed", "accumulate", "normalize") else "backward"]
         h = hashlib.sha1()
         for rel in src:
             with open(os.path.join(ROOT, rel), "rb") as f:
@@ -472,9 +472,11 @@ def implementation_bytes(kernel: str, n: int, px: int, c: int, s_feat: int, s_ou
     gs = c if c <= 2 else (c + 3) // 4 * 4
     nv = n if n_vis is None else n_vis
     return {
-        "clear": px * (8 + 4 + 4 * c),                          # write key, count, sums
+        "clear": px * 8,                                        # write key (with a seed pass; else count, sums too)
+        "seed": px * (8 + 4 + 4 * c) + nv * c * s_feat,         # key, the nearest points' tau -> count, sums
         "depth": n * (12 + 1) + px * 8 * 2,                     # read xyz -> layer byte; read+write keys
-        "accumulate": n * (12 + 1 + c * s_feat + 4) + px * (8 + 2 * (4 + 4 * c)),  # xyz, byte, tau -> mask; keys; RMW count+sums
+        # xyz, byte -> mask; keys (with a seed pass: the few others' tau and sums are not counted)
+        "accumulate": n * (12 + 1 + 4) + px * 8,
         "normalize": px * (4 + 4 * c + c * s_out),              # read count, sums; write image
         "bwd_prepass": px * (8 + 4 + 4 * c + 4 * c + 16 + 4 * gs),  # key, count, sums, G -> info, G'
         "bwd_bin": n * 8 + nv * 4 + 2 * bin_table,                    # masks twice -> list; table written, read

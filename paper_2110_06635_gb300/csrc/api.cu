@@ -326,7 +326,7 @@ adop_status render_chunk(const adop_points* pts, const adop_camera* cams, int k0
     return cuda_fail(e, "clear launch");
   if ((e = timed("depth", s, [&] { return launch_depth(lc, a, s); })) != cudaSuccess)
     return cuda_fail(e, "depth pass launch");
-  if ((e = timed("seed", s, [&] { return launch_seed(lc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
+  if (a.seeded && (e = timed("seed", s, [&] { return launch_seed(lc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
     return cuda_fail(e, "seed launch");
   if ((e = timed("accumulate", s, [&] { return launch_accum(lc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
     return cuda_fail(e, "accumulate launch");
@@ -586,7 +586,8 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
           return cuda_fail(e, "clear launch");
         if ((e = timed("depth", s, [&] { return launch_depth(rc, a, s); })) != cudaSuccess)
           return cuda_fail(e, "depth pass launch");
-        if ((e = timed("seed", s, [&] { return launch_seed(rc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
+        if (a.seeded &&
+            (e = timed("seed", s, [&] { return launch_seed(rc, a, pts->c, pts->feat_dtype, s); })) != cudaSuccess)
           return cuda_fail(e, "seed launch");
         if ((e = timed("accumulate", s, [&] { return launch_accum(rc, a, pts->c, pts->feat_dtype, s); })) !=
             cudaSuccess)
