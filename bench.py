@@ -312,7 +312,7 @@ def recorded_atomics(kernel: str):
 # bench name of each library kernel (the k_bin_* launches are one entry)
 NCU_KERNELS = {"k_clear": "clear", "k_depth": "depth", "k_seed": "seed", "k_accum": "accumulate", "k_normalize": "normalize",
                "k_bwd_prepass": "bwd_prepass", "k_bin_count_blk": "bwd_bin", "k_bin_scan": "bwd_bin",
-               "k_bin_scatter_blk": "bwd_bin", "k_bwd_items": "bwd_points", "k_bwd_reduce": "bwd_reduce"}
+               "k_bin_scatter_blk": "bwd_bin", "k_zero_grads": "bwd_zero", "k_bwd_items": "bwd_points", "k_bwd_reduce": "bwd_reduce"}
 NCU_SOURCES = {"forward": ["paper_2110_06635_gb300/csrc/forward.cu", "paper_2110_06635_gb300/csrc/adop_device.cuh"],
                "backward": ["paper_2110_06635_gb300/csrc/backward.cu", "paper_2110_06635_gb300/csrc/adop_device.cuh"]}
 

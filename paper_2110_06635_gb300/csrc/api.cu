@@ -623,6 +623,11 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
     if (bin &&
         (e = timed("bwd_bin", s, [&] { return launch_bin(lc, a, b, pts->c, s); })) != cudaSuccess)
       return cuda_fail(e, "backward binning launch");
+    b.zeroed = bin && mode == kGradAssign && zero_first(pts->n, lc.c[0].off[params->levels],
+                                                             pts->c * (b.feat_out == ADOP_F32 ? 4 : 2)) ? 1 : 0;
+    if (b.zeroed && (grad_feat || grad_xyz) &&
+        (e = timed("bwd_zero", s, [&] { return launch_zero_grads(b, pts->n, pts->c, s); })) != cudaSuccess)
+      return cuda_fail(e, "zero gradients launch");
     // the prepass and the point pass that reads its records, a few cameras at a time
     const int per = cams_per_backward(pts->n, nc);
     for (int j0 = 0; j0 < nc; j0 += per) {

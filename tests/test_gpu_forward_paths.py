@@ -110,6 +110,40 @@ def test_binned_gradient_buffers_only_aligned_as_asked(adop, dtype):
     assert unseen.any() and not got[0][0][unseen].any() and not got[0][1][unseen].any()
 
 
+@pytest.mark.parametrize("c,dtype", [(4, "f32"), (3, "f16")])
+def test_gradients_zeroed_ahead(adop, c, dtype):
+    """From 16M points on, eight per pixel, the zero gradients are written
+    ahead of the point pass: the same as gradients added onto zeros (FP32
+    rounding of sums in another order, one step of FP16), every point written
+    (buffers filled with NaN), dL/dx on a 16-byte boundary and off it."""
+    import torch
+    from parity import assert_close
+    n = (1 << 24) + 5
+    rng = np.random.default_rng(1)
+    xyz = torch.from_numpy(rng.random((n, 3), dtype=np.float32)).cuda()
+    feat = torch.from_numpy(rng.random((n, c), dtype=np.float32)).cuda()
+    cam = _camera(320, 200)
+    pts = adop.Points(xyz, feat)
+    params = adop.Params(4, 0.01, 1e-3, None, adop.ADOP_FLAG_GRAD_ASSIGN)
+    fr = adop.Frame.alloc(cam, c, 4, torch.float32, True, "cuda", n)
+    ws = adop.alloc_workspace(pts, [cam], params)
+    adop.adop_render_forward(pts, [cam], params, [fr], ws)
+    G = [[torch.from_numpy(g).cuda() for g in scenes.upstream_grad(cam.w, cam.h, 4, c, 8)]]
+    want = [torch.zeros((n, c), device="cuda"), torch.zeros((n, 3), device="cuda")]
+    adop.adop_render_backward(pts, [cam], adop.Params(4, 0.01, 1e-3, None, 0), [fr], G, *want, None, None, ws)
+    want = [w.cpu().numpy() for w in want]
+    seen = fr.vis.cpu().numpy() & 0xFF != 0
+    assert seen.any() and not seen.all()
+    for offset in (0, 1):
+        gx = torch.full((n * 3 + 4,), float("nan"), device="cuda")[offset:offset + n * 3].view(n, 3)
+        gf = torch.full((n, c), float("nan"), dtype=torch.float16 if dtype == "f16" else torch.float32, device="cuda")
+        adop.adop_render_backward(pts, [cam], params, [fr], G, gf, gx, None, None, ws)
+        gf, gx = gf.float().cpu().numpy(), gx.cpu().numpy()
+        assert not gf[~seen].any() and not gx[~seen].any()
+        assert_close(gf[seen], want[0][seen], 1e-6 if dtype == "f32" else 2e-3, "dL/dtau")
+        assert_close(gx[seen], want[1][seen], 1e-5, "dL/dx")
+
+
 def test_layer_masks_only_4_byte_aligned(adop):
     import torch
     sc = scenes.tiny_spheres(2_334_731, 4, seed=5)
