@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256) k_query(int64_t n, int k, Grid g, const u
       }
       const float4 q = __ldg(sorted + s);
       const float d2 = dist2(q.x - p.x, q.y - p.y, q.z - p.z);
-      best.insert((__float_as_uint(q.w) == tag && s != (uint32_t)i) ? d2 : INFINITY);
+      best.insert((__float_as_uint(q.w) == tag && s != (uint32_t)i) ? fminf(d2, INFINITY) : INFINITY);  // (NaN: no neighbour)
       ++s;
     }
     const float kth = best.kth(k);
