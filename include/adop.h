@@ -429,9 +429,12 @@ int32_t adop_profile_collect(adop_kernel_stat* out, int32_t max);
  * distance to its k-th nearest other point (the paper uses k = 4), by a
  * uniform-grid search on the GPU with cells of 1.5x the median k-NN distance
  * of 256 sampled points; +inf if the cloud has fewer than k + 1 points.
- * Exact (FP32 distances) when the k-th neighbour lies within 8 cells and at
- * most 65536 candidates are scanned for the point; otherwise an upper bound
- * (isolated outliers, which discarding keeps anyway).  xyz: n x 3 FP32
+ * Exact (FP32 distances) when the k-th neighbour lies within 8 cells; otherwise
+ * an upper bound (isolated outliers, which discarding keeps anyway).  Where
+ * the cells around a point hold more than 65536 candidates the search is
+ * repeated for it on cells an eighth as wide (but no less than 2^-20 of the
+ * box), from the nearest outwards, and is exact there too unless another 65536
+ * candidates do not reach the k-th neighbour.  xyz: n x 3 FP32
  * (device); radius: n FP32 (device, output); 1 <= k <= 16.  A preprocess: it
  * synchronises `stream` once (to size the grid).  Workspace from
  * adop_point_radius_workspace_bytes(n).

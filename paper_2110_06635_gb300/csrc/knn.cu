@@ -9,8 +9,11 @@
 //   3. counting sort of the points by the hash of their search cell (1.6 h)
 //   4. per point, in sorted order: the 8 search cells nearest to it (k_query);
 //      points that these do not settle search a wider cube (k_query_far)
+//   5. points whose search cells hold too many candidates: steps 3 and 4 again
+//      for them alone, on cells of h / 8, nearest cells first (k_query_dense)
 // 5M points on 50 surfaces: 8.73 ms with one block per sample and the points
 // queried in input order cell by cell, 1.12 ms now.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -326,8 +329,9 @@ __device__ __forceinline__ uint32_t cell_tag(int Cx, int Cy, int Cz) {
 // that their round trips overlap.
 constexpr int kAhead = 4;
 
-__global__ void __launch_bounds__(256) k_count(const float* __restrict__ xyz, int64_t n, Grid g,
-                                               uint2* __restrict__ bkt, uint32_t* __restrict__ count) {
+// (The sort's steps read with plain loads what the step before wrote: they also
+// run one after the other within k_query_dense.)
+__device__ __forceinline__ void count_points(const float* xyz, int64_t n, const Grid& g, uint2* bkt, uint32_t* count) {
   const int64_t S = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kAhead * S) {
     uint32_t b[kAhead], rank[kAhead];
@@ -347,38 +351,21 @@ __global__ void __launch_bounds__(256) k_count(const float* __restrict__ xyz, in
   }
 }
 
-// Exclusive scan of `count` (length m) into `start` (length m + 1), three
-// phases over tiles of 4096 entries.
-constexpr int kScanTile = 4096;
-
-__global__ void __launch_bounds__(1024) k_scan_tiles(const uint32_t* __restrict__ count, int64_t m,
-                                                     uint32_t* __restrict__ tile_sum) {
-  __shared__ uint32_t warp_sum[32];
-  const int64_t t0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * 4;
-  uint32_t s = 0;
-  for (int q = 0; q < 4; ++q)
-    if (t0 + q < m) s += count[t0 + q];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    uint32_t v = warp_sum[threadIdx.x];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (threadIdx.x == 0) tile_sum[blockIdx.x] = v;
-  }
+__global__ void __launch_bounds__(256) k_count(const float* __restrict__ xyz, int64_t n, Grid g,
+                                               uint2* __restrict__ bkt, uint32_t* __restrict__ count) {
+  count_points(xyz, n, g, bkt, count);
 }
 
-__global__ void __launch_bounds__(1024) k_scan_sums(uint32_t* __restrict__ tile_sum, int64_t tiles) {
-  // single block: exclusive scan of the tile sums, serial chunks per thread
-  __shared__ uint32_t warp_sum[32];
-  const int64_t per = (tiles + 1023) / 1024;
-  const int64_t a = threadIdx.x * per, b = min(tiles, a + per);
-  uint32_t local = 0;
-  for (int64_t t = a; t < b; ++t) local += tile_sum[t];
+// Exclusive scan of `count` (length m) into `start` (length m + 1), three
+// phases over tiles of 4096 entries, by blocks of T threads.
+constexpr int kScanTile = 4096;
+
+// This thread's exclusive prefix of v over its block.
+template <int T>
+__device__ __forceinline__ uint32_t block_prefix(uint32_t v) {
+  __shared__ uint32_t warp_sum[T / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t incl = local;
+  uint32_t incl = v;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -387,16 +374,39 @@ __global__ void __launch_bounds__(1024) k_scan_sums(uint32_t* __restrict__ tile_
   if (lane == 31) warp_sum[warp] = incl;
   __syncthreads();
   if (warp == 0) {
-    uint32_t w = warp_sum[lane];
+    uint32_t w = lane < T / 32 ? warp_sum[lane] : 0u;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
-    warp_sum[lane] = w;
+    if (lane < T / 32) warp_sum[lane] = w;
   }
   __syncthreads();
-  uint32_t run = incl - local + (warp > 0 ? warp_sum[warp - 1] : 0u);
+  const uint32_t before = incl - v + (warp > 0 ? warp_sum[warp - 1] : 0u);
+  __syncthreads();  // (the block may call again)
+  return before;
+}
+
+template <int T>
+__device__ __forceinline__ void scan_tile(const uint32_t* count, int64_t m, int64_t tile, uint32_t* tile_sum) {
+  const int64_t t0 = tile * kScanTile + threadIdx.x * (kScanTile / T);
+  uint32_t s = 0;
+#pragma unroll
+  for (int q = 0; q < kScanTile / T; ++q)
+    if (t0 + q < m) s += count[t0 + q];
+  const uint32_t before = block_prefix<T>(s);
+  if (threadIdx.x == T - 1) tile_sum[tile] = before + s;
+}
+
+// one block: exclusive scan of the tile sums, serial chunks per thread
+template <int T>
+__device__ __forceinline__ void scan_sums(uint32_t* tile_sum, int64_t tiles) {
+  const int64_t per = (tiles + T - 1) / T;
+  const int64_t a = threadIdx.x * per, b = min(tiles, a + per);
+  uint32_t local = 0;
+  for (int64_t t = a; t < b; ++t) local += tile_sum[t];
+  uint32_t run = block_prefix<T>(local);
   for (int64_t t = a; t < b; ++t) {
     const uint32_t v = tile_sum[t];
     tile_sum[t] = run;
@@ -404,47 +414,45 @@ __global__ void __launch_bounds__(1024) k_scan_sums(uint32_t* __restrict__ tile_
   }
 }
 
-__global__ void __launch_bounds__(1024) k_scan_apply(const uint32_t* __restrict__ count, int64_t m,
-                                                     const uint32_t* __restrict__ tile_off, uint32_t* __restrict__ start,
-                                                     uint32_t total) {
-  __shared__ uint32_t warp_sum[32];
-  const int64_t t0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * 4;
-  uint32_t v[4], s = 0;
-  for (int q = 0; q < 4; ++q) {
+// (Leaves `count` cleared, for a second sort.)
+template <int T>
+__device__ __forceinline__ void scan_apply(uint32_t* count, int64_t m, int64_t tile, const uint32_t* tile_off,
+                                           uint32_t* start, uint32_t total) {
+  const int64_t t0 = tile * kScanTile + threadIdx.x * (kScanTile / T);
+  uint32_t v[kScanTile / T], s = 0;
+#pragma unroll
+  for (int q = 0; q < kScanTile / T; ++q) {
     v[q] = t0 + q < m ? count[t0 + q] : 0u;
+    if (v[q]) count[t0 + q] = 0u;
     s += v[q];
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t incl = s;
+  uint32_t run = tile_off[tile] + block_prefix<T>(s);
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) warp_sum[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = warp_sum[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += y;
-    }
-    warp_sum[lane] = w;
-  }
-  __syncthreads();
-  uint32_t run = tile_off[blockIdx.x] + incl - s + (warp > 0 ? warp_sum[warp - 1] : 0u);
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < kScanTile / T; ++q)
     if (t0 + q < m) {
       start[t0 + q] = run;
       run += v[q];
     }
-  if (blockIdx.x == 0 && threadIdx.x == 0) start[m] = total;
+  if (tile == 0 && threadIdx.x == 0) start[m] = total;
 }
 
-__global__ void __launch_bounds__(256) k_scatter(const float* __restrict__ xyz, int64_t n, Grid g,
-                                                 const uint2* __restrict__ bkt, const uint32_t* __restrict__ start,
-                                                 float4* __restrict__ sorted, uint32_t* __restrict__ index) {
+__global__ void __launch_bounds__(1024) k_scan_tiles(const uint32_t* __restrict__ count, int64_t m,
+                                                     uint32_t* __restrict__ tile_sum) {
+  scan_tile<1024>(count, m, blockIdx.x, tile_sum);
+}
+
+__global__ void __launch_bounds__(1024) k_scan_sums(uint32_t* __restrict__ tile_sum, int64_t tiles) {
+  scan_sums<1024>(tile_sum, tiles);
+}
+
+__global__ void __launch_bounds__(1024) k_scan_apply(uint32_t* __restrict__ count, int64_t m,
+                                                     const uint32_t* __restrict__ tile_off, uint32_t* __restrict__ start,
+                                                     uint32_t total) {
+  scan_apply<1024>(count, m, blockIdx.x, tile_off, start, total);
+}
+
+__device__ __forceinline__ void scatter_points(const float* xyz, int64_t n, const Grid& g, const uint2* bkt,
+                                               const uint32_t* start, float4* sorted, uint32_t* index) {
   const int64_t S = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kAhead * S) {
     uint2 b[kAhead];
@@ -453,13 +461,13 @@ __global__ void __launch_bounds__(256) k_scatter(const float* __restrict__ xyz, 
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
       const int64_t i = min(i0 + u * S, n - 1);
-      b[u] = __ldg(bkt + i);
+      b[u] = bkt[i];
       p[u].x = __ldg(xyz + 3 * i);
       p[u].y = __ldg(xyz + 3 * i + 1);
       p[u].z = __ldg(xyz + 3 * i + 2);
     }
 #pragma unroll
-    for (int u = 0; u < kAhead; ++u) pos[u] = __ldg(start + b[u].x) + b[u].y;
+    for (int u = 0; u < kAhead; ++u) pos[u] = start[b[u].x] + b[u].y;
 #pragma unroll
     for (int u = 0; u < kAhead; ++u) {
       if (i0 + u * S >= n) continue;
@@ -472,14 +480,29 @@ __global__ void __launch_bounds__(256) k_scatter(const float* __restrict__ xyz, 
   }
 }
 
+__global__ void __launch_bounds__(256) k_scatter(const float* __restrict__ xyz, int64_t n, Grid g,
+                                                 const uint2* __restrict__ bkt, const uint32_t* __restrict__ start,
+                                                 float4* __restrict__ sorted, uint32_t* __restrict__ index) {
+  scatter_points(xyz, n, g, bkt, start, sorted, index);
+}
+
 // The search is bounded: a point's result is the k-th smallest distance to
 // the points at most kMaxRing cells away along each axis (+inf if there are
 // fewer than k) -- the exact result unless the true neighbour is further than
-// that, else an upper bound -- and at most kMaxScan candidates are looked at
-// (a cell with more copies of one place than that), past which the k-th
-// smallest found so far stands.
+// that, else an upper bound.  k_query looks at kMaxScan candidates at most and
+// each lane of k_query_far at as many per ball; a point that has more is
+// searched again by k_query_dense, on cells of h / kFine from the nearest
+// outwards, and only there, after another kMaxScan candidates, does the
+// smallest found so far stand (more points than that in cells of h / kFine, or
+// of 2^-20 of the box where that is wider, around a point that are no copies
+// of it).
 constexpr int kMaxRing = 8;
 constexpr int kMaxScan = 1 << 16;
+constexpr float kFine = 8.0f;
+
+// What is left: points listed for k_query_far, listed for k_query_dense, and
+// passed on to it by k_query_far.
+enum Counts { kListed = 0, kDense = 1, kMarked = 2 };
 
 // The K smallest squared distances met, ascending; +inf where there are fewer.
 template <int K>
@@ -520,7 +543,7 @@ template <int K>
 __global__ void __launch_bounds__(256) k_query(int64_t n, int k, Grid g, const uint32_t* __restrict__ start,
                                                const float4* __restrict__ sorted,
                                                const uint32_t* __restrict__ index, float* __restrict__ radius,
-                                               uint32_t* __restrict__ pending, uint32_t* __restrict__ pending_count) {
+                                               uint32_t* __restrict__ pending, uint32_t* __restrict__ counts) {
   __shared__ uint2 s_range[8][256];  // first point, count and octant
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -566,8 +589,15 @@ __global__ void __launch_bounds__(256) k_query(int64_t n, int k, Grid g, const u
     }
     const float kth = best.kth(k);
     const float reach = fmaxf(1.0f - near - g.slack, 0.0f);
-    radius[__ldg(index + i)] = sqrtf(kth);
-    if (kth > reach * reach * g.s2_low && scanned < kMaxScan) pending[atomicAdd(pending_count, 1u)] = (uint32_t)i;
+    const uint32_t at = __ldg(index + i);
+    radius[at] = sqrtf(kth);
+    // too many candidates: what was found is the best of a part of them.  These
+    // points are listed from the end of `pending`, by their place in xyz
+    if (scanned >= kMaxScan) {
+      if (kth > 0.0f) pending[n - 1 - atomicAdd(counts + kDense, 1u)] = at;
+    } else if (kth > reach * reach * g.s2_low) {
+      pending[atomicAdd(counts + kListed, 1u)] = (uint32_t)i;
+    }
   }
 }
 
@@ -577,13 +607,15 @@ __global__ void __launch_bounds__(256) k_query(int64_t n, int k, Grid g, const u
 // or 4 h and 9 h (past which nothing counts) while fewer than k points were
 // found.  (A thread each took 188 us on 5M points: few threads, each a chain
 // of some 27 lookups.)
+constexpr uint32_t kMark = 0x80000000u;
+constexpr int kDenseBlocksPerSm = 4;  // resident: 64 registers a thread
+
 template <int K>
-__global__ void __launch_bounds__(256) k_query_far(int k, Grid g, const uint32_t* __restrict__ start,
-                                                   const float4* __restrict__ sorted,
-                                                   const uint32_t* __restrict__ index, int max_ring,
-                                                   float* __restrict__ radius, const uint32_t* __restrict__ pending,
-                                                   const uint32_t* __restrict__ pending_count) {
-  const uint32_t count = *pending_count;
+__global__ void __launch_bounds__(256, K == 4 ? 5 : 4)
+    k_query_far(int k, Grid g, const uint32_t* __restrict__ start, const float4* __restrict__ sorted,
+                const uint32_t* __restrict__ index, int max_ring, float* __restrict__ radius,
+                uint32_t* __restrict__ pending, uint32_t* __restrict__ counts) {
+  const uint32_t count = counts[kListed];
   const int rings = min(max_ring, kMaxRing);
   const int lane = threadIdx.x & 31;
   const uint32_t warps = gridDim.x * (blockDim.x >> 5);
@@ -594,9 +626,10 @@ __global__ void __launch_bounds__(256) k_query_far(int k, Grid g, const uint32_t
     int cx, cy, cz;
     cell_of(g, g.inv_h, p.x, p.y, p.z, cx, cy, cz);
     const float fx = (p.x - g.ox) * g.inv_s, fy = (p.y - g.oy) * g.inv_s, fz = (p.z - g.oz) * g.inv_s;
-    float found = radius[at];  // an upper bound of the result, or +inf
+    const float before = radius[at];  // an upper bound of the result, or +inf
+    float found = before;
     const float most = (float)(rings + 1) / kSearch + g.slack;  // search cells that the cube of +-rings cells spans
-    bool last;
+    bool last, full = false;
     float ball = 0.0f;
     do {
       if (found < INFINITY) {
@@ -649,9 +682,131 @@ __global__ void __launch_bounds__(256) k_query_far(int k, Grid g, const uint32_t
       found = sqrtf(kth);
       // the k-th of a first, smaller ball is exact if the ball reaches it
       if (found < INFINITY && found * g.inv_s * 1.00001f + g.slack <= ball) last = true;
-      if (__any_sync(0xffffffffu, scanned >= kMaxScan)) last = true;
-    } while (!last);
-    if (lane == 0) radius[at] = found;
+      full = __any_sync(0xffffffffu, scanned >= kMaxScan);
+    } while (!last && !full);
+    if (lane == 0) {
+      radius[at] = full ? fminf(found, before) : found;
+      if (full) {  // (the point's place in xyz, marked: n < 2^31)
+        pending[j] = at | kMark;
+        atomicAdd(counts + kMarked, 1u);
+      }
+    }
+  }
+}
+
+// The points with too many candidates, a warp each, over all points sorted
+// again by cells of h / kFine: the cells around the point in shells, nearest
+// first, a cell a lane to look up and the whole warp over each cell's points,
+// until the k-th distance found is within the shells (or a shell is past what
+// is known already: radius holds the best of the first search, or +inf).
+// Sort and search are one cooperative launch, which ends at once where there
+// is no such point: six launches that end at once cost 27 us of a call on a
+// thousand points (131 us), and asking on the host would be a second
+// synchronisation.
+template <int K>
+__global__ void __launch_bounds__(256, kDenseBlocksPerSm)
+    k_query_dense(const float* __restrict__ xyz, int64_t n, int k, Grid g, float most, uint2* bkt, uint32_t* count,
+                  int64_t m, uint32_t* tiles, uint32_t* start, float4* sorted, uint32_t* index,
+                  float* __restrict__ radius, const uint32_t* __restrict__ pending,
+                  const uint32_t* __restrict__ counts) {
+  if ((counts[kDense] | counts[kMarked]) == 0u) return;  // (every block alike)
+  {
+    const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+    const int64_t nt = (m + kScanTile - 1) / kScanTile;
+    count_points(xyz, n, g, bkt, count);
+    grid.sync();
+    for (int64_t t = blockIdx.x; t < nt; t += gridDim.x) scan_tile<256>(count, m, t, tiles);
+    grid.sync();
+    if (blockIdx.x == 0) scan_sums<256>(tiles, nt);
+    grid.sync();
+    for (int64_t t = blockIdx.x; t < nt; t += gridDim.x) scan_apply<256>(count, m, t, tiles, start, (uint32_t)n);
+    grid.sync();
+    scatter_points(xyz, n, g, bkt, start, sorted, index);
+    grid.sync();
+  }
+  const uint32_t listed = counts[kListed], total = listed + counts[kDense];  // <= n < 2^31
+  const int lane = threadIdx.x & 31;
+  const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+  for (uint32_t j = (counts[kMarked] ? 0u : listed) + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < total;
+       j += warps) {  // warp-uniform
+    const uint32_t entry = j < listed ? pending[j] : pending[n - 1 - (j - listed)] | kMark;
+    if (!(entry & kMark)) continue;  // settled by k_query_far
+    const int64_t at = entry & ~kMark;
+    const float px = __ldg(xyz + 3 * at), py = __ldg(xyz + 3 * at + 1), pz = __ldg(xyz + 3 * at + 2);
+    const uint2 own_slot = bkt[at];
+    const uint32_t own = start[own_slot.x] + own_slot.y;
+    int cx, cy, cz;
+    cell_of(g, g.inv_s, px, py, pz, cx, cy, cz);
+    const float fx = (px - g.ox) * g.inv_s, fy = (py - g.oy) * g.inv_s, fz = (pz - g.oz) * g.inv_s;
+    const float known = radius[at];
+    const float ball = known < INFINITY ? fminf(known * g.inv_s * 1.00001f + g.slack, most) : most;
+    float limit = known < INFINITY ? known * known * 1.00001f : INFINITY;  // no further point counts
+    float kth = INFINITY;
+    int scanned = 0;
+    Nearest<K> best;
+    best.clear();
+    for (int r = 0;; ++r) {
+      const int side = 2 * r + 1, faces = 2 * side * side, layer = 8 * r;
+      const int cells = r == 0 ? 1 : faces + (side - 2) * layer;
+      for (int c0 = 0; c0 < cells && scanned < kMaxScan; c0 += 32) {
+        int c = c0 + lane, dx = 0, dy = 0, dz = 0;
+        if (r > 0 && c < faces) {  // the two faces across z
+          dz = c < side * side ? -r : r;
+          c = c < side * side ? c : c - side * side;
+          dx = c % side - r;
+          dy = c / side - r;
+        } else if (r > 0 && c < cells) {  // the layers between them: four edges of 2 r cells
+          c -= faces;
+          dz = c / layer - (r - 1);
+          const int edge = c % layer / (2 * r), o = c % (2 * r) - r;
+          dx = edge == 0 ? o : (edge == 1 ? r : (edge == 2 ? -o : -r));
+          dy = edge == 0 ? -r : (edge == 1 ? o : (edge == 2 ? r : -o));
+        }
+        const int qx = cx + dx, qy = cy + dy, qz = cz + dz;
+        const float ex = fmaxf(fmaxf((float)qx - fx, fx - (float)(qx + 1)) - g.slack, 0.0f);
+        const float ey = fmaxf(fmaxf((float)qy - fy, fy - (float)(qy + 1)) - g.slack, 0.0f);
+        const float ez = fmaxf(fmaxf((float)qz - fz, fz - (float)(qz + 1)) - g.slack, 0.0f);
+        uint32_t s = 0, len = 0;
+        if (c0 + lane < cells && !((ex * ex + ey * ey + ez * ez) * g.s2_low > limit)) {
+          const uint32_t b = bucket(g, qx, qy, qz);
+          s = start[b];
+          len = start[b + 1] - s;
+        }
+        const uint32_t tag = cell_tag(qx, qy, qz);
+        for (unsigned m = __ballot_sync(0xffffffffu, len > 0u); m && scanned < kMaxScan; m &= m - 1u) {
+          const int src = __ffs(m) - 1;
+          const uint32_t first = __shfl_sync(0xffffffffu, s, src), want = __shfl_sync(0xffffffffu, tag, src);
+          const uint32_t take = min(__shfl_sync(0xffffffffu, len, src), (uint32_t)(kMaxScan - scanned));
+          scanned += (int)take;
+          for (uint32_t t = lane; t < take; t += 32) {
+            const float4 q = sorted[first + t];
+            const float d2 = dist2(q.x - px, q.y - py, q.z - pz);
+            if (d2 < best.d[K - 1] && __float_as_uint(q.w) == want && first + t != own) best.insert(d2);
+          }
+          __syncwarp();
+        }
+      }
+      // the k-th smallest so far; the k smallest stay, one in each of the first k lanes
+      float mine = INFINITY;
+      for (int q = 0; q < k; ++q) {
+        const uint32_t head = __float_as_uint(best.d[0]);
+        const uint32_t least = __reduce_min_sync(0xffffffffu, head);
+        const unsigned who = __ballot_sync(0xffffffffu, head == least);
+        if (lane == __ffs(who) - 1) {
+#pragma unroll
+          for (int i = 0; i < K - 1; ++i) best.d[i] = best.d[i + 1];
+          best.d[K - 1] = INFINITY;
+        }
+        kth = __uint_as_float(least);
+        if (lane == q) mine = kth;
+      }
+      best.clear();
+      best.d[0] = mine;
+      limit = fminf(limit, kth * 1.00001f);
+      const float reach = fmaxf((float)r - g.slack, 0.0f);
+      if (kth <= reach * reach * g.s2_low || (float)r >= ball || scanned >= kMaxScan) break;
+    }
+    if (lane == 0) radius[at] = fminf(known, sqrtf(kth));
   }
 }
 
@@ -676,7 +831,7 @@ Layout layout(int64_t n) {
   L.groups = std::min(total, std::max((int64_t)kSubLeast / kSubGroup, total / 128));
   L.scan = L.groups < total;
   size_t o = 0;
-  L.box = o;         o = up(o + 7 * 4);  // and the count of pending
+  L.box = o;         o = up(o + 9 * 4);  // and Counts
   L.samples = o;     o = up(o + kSamples * 4);
   L.bound = o;       o = up(o + kSamples * 4);
   L.list_count = o;  o = up(o + kSamples * 4);
@@ -736,7 +891,7 @@ adop_status adop_point_radius(const float* xyz, int64_t n, int32_t k, float* rad
   const int blocks = adop::num_sms() * 8;
   cudaError_t e;
   if ((e = cudaMemsetAsync(box, 0xff, 3 * 4, s)) != cudaSuccess ||
-      (e = cudaMemsetAsync(box + 3, 0, 4 * 4, s)) != cudaSuccess)
+      (e = cudaMemsetAsync(box + 3, 0, 6 * 4, s)) != cudaSuccess)
     return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   k_bbox<<<blocks, 256, 0, s>>>(xyz, n, box);
   k_sample_bound<<<kSamples, kBoundThreads, 0, s>>>(xyz, n, k, L.groups, bound, list_count);
@@ -774,9 +929,11 @@ adop_status adop_point_radius(const float* xyz, int64_t n, int32_t k, float* rad
   h = std::max({h, extent / 1048576.0f, 1e-20f});
   if (v.empty()) h = std::max(extent, 1e-20f);  // fewer than k + 1 points
   const int max_ring = (int)std::ceil(extent / h) + 2;
-  const float cell = h * kSearch;
-  const Grid g{lo[0], lo[1], lo[2], 1.0f / h, 1.0f / cell, cell * cell * 0.99998f, extent / cell * 5e-7f + 1e-6f,
-               (uint32_t)(L.m - 1)};
+  auto grid_of = [&](float cell) {  // the sorted cells' size
+    return Grid{lo[0], lo[1], lo[2], 1.0f / h, 1.0f / cell, cell * cell * 0.99998f, extent / cell * 5e-7f + 1e-6f,
+                (uint32_t)(L.m - 1)};
+  };
+  const Grid g = grid_of(h * kSearch);
   if ((e = cudaMemsetAsync(count, 0, (size_t)L.m * 4, s)) != cudaSuccess) return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   k_count<<<blocks, 256, 0, s>>>(xyz, n, g, bkt, count);
   const int64_t nt = (L.m + kScanTile - 1) / kScanTile;
@@ -785,14 +942,26 @@ adop_status adop_point_radius(const float* xyz, int64_t n, int32_t k, float* rad
   k_scan_apply<<<(unsigned)nt, 1024, 0, s>>>(count, L.m, tiles, start, (uint32_t)n);
   k_scatter<<<blocks, 256, 0, s>>>(xyz, n, g, bkt, start, sorted, index);
   const unsigned qblocks = (unsigned)std::min((n + 255) / 256, (int64_t)blocks * 8);
-  uint32_t* pending_count = box + 6;
+  uint32_t* counts = box + 6;
   if (k == 4) {
-    k_query<4><<<qblocks, 256, 0, s>>>(n, k, g, start, sorted, index, radius, pending, pending_count);
-    k_query_far<4><<<blocks, 256, 0, s>>>(k, g, start, sorted, index, max_ring, radius, pending, pending_count);
+    k_query<4><<<qblocks, 256, 0, s>>>(n, k, g, start, sorted, index, radius, pending, counts);
+    k_query_far<4><<<blocks, 256, 0, s>>>(k, g, start, sorted, index, max_ring, radius, pending, counts);
   } else {
-    k_query<kMaxK><<<qblocks, 256, 0, s>>>(n, k, g, start, sorted, index, radius, pending, pending_count);
-    k_query_far<kMaxK><<<blocks, 256, 0, s>>>(k, g, start, sorted, index, max_ring, radius, pending, pending_count);
+    k_query<kMaxK><<<qblocks, 256, 0, s>>>(n, k, g, start, sorted, index, radius, pending, counts);
+    k_query_far<kMaxK><<<blocks, 256, 0, s>>>(k, g, start, sorted, index, max_ring, radius, pending, counts);
   }
+  const float fine = std::max({h / kFine, extent / 1048576.0f, 1e-20f});
+  Grid gf = grid_of(fine);
+  float most = (float)(std::min(max_ring, kMaxRing) + 1) * (h / fine) + gf.slack;
+  void* args[] = {(void*)&xyz, &n, &k, &gf, &most, &bkt, &count, (void*)&L.m, &tiles, &start, &sorted, &index, &radius,
+                  &pending, &counts};
+  const void* dense = k == 4 ? (const void*)k_query_dense<4> : (const void*)k_query_dense<kMaxK>;
+  for (int grid = adop::num_sms() * kDenseBlocksPerSm;; grid /= 2) {  // (fewer where only a part of the SMs is ours)
+    e = cudaLaunchCooperativeKernel(dense, dim3(grid), dim3(256), args, 0, s);
+    if (e != cudaErrorCooperativeLaunchTooLarge || grid < 2) break;
+    cudaGetLastError();
+  }
+  if (e != cudaSuccess) return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   if ((e = cudaGetLastError()) != cudaSuccess) return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
   return ADOP_OK;
 }
