@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -930,8 +931,9 @@ adop_status adop_point_radius(const float* xyz, int64_t n, int32_t k, float* rad
   if (v.empty()) h = std::max(extent, 1e-20f);  // fewer than k + 1 points
   const int max_ring = (int)std::ceil(extent / h) + 2;
   auto grid_of = [&](float cell) {  // the sorted cells' size
-    return Grid{lo[0], lo[1], lo[2], 1.0f / h, 1.0f / cell, cell * cell * 0.99998f, extent / cell * 5e-7f + 1e-6f,
-                (uint32_t)(L.m - 1)};
+    // (the square stays finite: 0 x inf would compare as no bound at all)
+    return Grid{lo[0], lo[1], lo[2], 1.0f / h, 1.0f / cell, std::min(cell * cell * 0.99998f, FLT_MAX),
+                extent / cell * 5e-7f + 1e-6f, (uint32_t)(L.m - 1)};
   };
   const Grid g = grid_of(h * kSearch);
   if ((e = cudaMemsetAsync(count, 0, (size_t)L.m * 4, s)) != cudaSuccess) return fail(ADOP_ERR_CUDA, cudaGetErrorString(e));
