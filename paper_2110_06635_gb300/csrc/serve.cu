@@ -103,6 +103,7 @@ struct Server {
   std::vector<std::unique_ptr<Batch>> inflight;
   uint64_t next_ticket = 1;
   int active = 0;                   // admitted + launched requests (slots in use)
+  size_t state_sum = 0, bytes_sum = 0;  // over them: pixel state, a byte per point of the cloud
   bool stop = false;
   std::thread worker;
 
@@ -119,6 +120,8 @@ struct Server {
     alloc.release(r.offset);
     if (r.early != SIZE_MAX) alloc.release(r.early);
     r.offset = r.early = SIZE_MAX;
+    state_sum -= alloc.round(r.bytes);
+    bytes_sum -= alloc.round((size_t)clouds[r.cloud].n);
   }
   void reap_locked();
   void admit_locked();
@@ -155,16 +158,17 @@ void Server::admit_locked() {
     const size_t off = alloc.alloc(r.bytes);
     if (off == SIZE_MAX) break;  // strict FIFO: the head waits for memory
     r.offset = off;
-    // a byte per point lets the accumulate pass skip what the depth pass ruled
-    // out (sixteen requests over 8M points: 3.08 -> 2.71 ms); taken where the
-    // pool would hold eight such requests, so that it costs no concurrency
-    // where the pool is small
-    const size_t n = (size_t)clouds[r.cloud].n;
-    if (8 * (alloc.round(r.bytes) + alloc.round(n)) <= alloc.capacity()) r.early = alloc.alloc(n);
     r.state = kAdmitted;
     admitted.push_back(r.ticket);
     queue.pop();
     ++active;
+    // a byte per point lets the accumulate pass skip what the depth pass ruled
+    // out (sixteen requests over 8M points: 3.08 -> 2.71 ms)
+    const size_t n = (size_t)clouds[r.cloud].n;
+    state_sum += alloc.round(r.bytes);
+    bytes_sum += alloc.round(n);
+    const size_t run = std::min((size_t)cfg.max_slots, streams.size() * (size_t)cfg.max_batch);
+    if (bytes_cost_no_request(alloc.capacity(), run, (size_t)active, state_sum, bytes_sum)) r.early = alloc.alloc(n);
   }
 }
 

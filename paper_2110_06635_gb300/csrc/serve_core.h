@@ -81,6 +81,20 @@ class RangeAllocator {
   std::map<size_t, size_t> live_;  // offset -> length
 };
 
+// Whether an admitted request may also take its cloud's byte per point (which
+// the depth pass leaves for the accumulate pass) from the pool.  It must cost
+// no concurrency: of requests like those admitted, as many as can run at once
+// (`run`: streams x cameras per launch, or the slots) and fit the pool without
+// the bytes still fit with them.  `state` and `bytes` are the sums of the
+// pixel states and of the clouds' bytes over the `active` admitted requests,
+// this one among them.  (Where eight such requests had to fit, whatever could
+// run, 640x480 views of a 120M-point cloud filled a 1.2 GB pool thirteen at a
+// time, 66 without the bytes.)
+inline bool bytes_cost_no_request(size_t capacity, size_t run, size_t active, size_t state, size_t bytes) {
+  const size_t fit = std::min(run, capacity * active / state);
+  return fit * (state + bytes) <= capacity * active;
+}
+
 // Latency samples (milliseconds) and percentiles by nearest rank.
 class LatencyStats {
  public:
