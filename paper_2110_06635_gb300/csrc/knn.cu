@@ -415,16 +415,14 @@ __device__ __forceinline__ void scan_sums(uint32_t* tile_sum, int64_t tiles) {
   }
 }
 
-// (Leaves `count` cleared, for a second sort.)
 template <int T>
-__device__ __forceinline__ void scan_apply(uint32_t* count, int64_t m, int64_t tile, const uint32_t* tile_off,
+__device__ __forceinline__ void scan_apply(const uint32_t* count, int64_t m, int64_t tile, const uint32_t* tile_off,
                                            uint32_t* start, uint32_t total) {
   const int64_t t0 = tile * kScanTile + threadIdx.x * (kScanTile / T);
   uint32_t v[kScanTile / T], s = 0;
 #pragma unroll
   for (int q = 0; q < kScanTile / T; ++q) {
     v[q] = t0 + q < m ? count[t0 + q] : 0u;
-    if (v[q]) count[t0 + q] = 0u;
     s += v[q];
   }
   uint32_t run = tile_off[tile] + block_prefix<T>(s);
@@ -446,7 +444,7 @@ __global__ void __launch_bounds__(1024) k_scan_sums(uint32_t* __restrict__ tile_
   scan_sums<1024>(tile_sum, tiles);
 }
 
-__global__ void __launch_bounds__(1024) k_scan_apply(uint32_t* __restrict__ count, int64_t m,
+__global__ void __launch_bounds__(1024) k_scan_apply(const uint32_t* __restrict__ count, int64_t m,
                                                      const uint32_t* __restrict__ tile_off, uint32_t* __restrict__ start,
                                                      uint32_t total) {
   scan_apply<1024>(count, m, blockIdx.x, tile_off, start, total);
@@ -607,12 +605,14 @@ __global__ void __launch_bounds__(256) k_query(int64_t n, int k, Grid g, const u
 // meets, its radius the distance found so far (every nearer point is in it),
 // or 4 h and 9 h (past which nothing counts) while fewer than k points were
 // found.  (A thread each took 188 us on 5M points: few threads, each a chain
-// of some 27 lookups.)
+// of some 27 lookups.)  64 registers, 4 blocks per SM: with the 48 and 56 that
+// the compiler settles on under other bounds the loop over a cell's points was
+// slower (1M points of a curve 580 and 571 us, now 538).
 constexpr uint32_t kMark = 0x80000000u;
 constexpr int kDenseBlocksPerSm = 4;  // resident: 64 registers a thread
 
 template <int K>
-__global__ void __launch_bounds__(256, K == 4 ? 5 : 4)
+__global__ void __launch_bounds__(256, 4)
     k_query_far(int k, Grid g, const uint32_t* __restrict__ start, const float4* __restrict__ sorted,
                 const uint32_t* __restrict__ index, int max_ring, float* __restrict__ radius,
                 uint32_t* __restrict__ pending, uint32_t* __restrict__ counts) {
@@ -627,10 +627,9 @@ __global__ void __launch_bounds__(256, K == 4 ? 5 : 4)
     int cx, cy, cz;
     cell_of(g, g.inv_h, p.x, p.y, p.z, cx, cy, cz);
     const float fx = (p.x - g.ox) * g.inv_s, fy = (p.y - g.oy) * g.inv_s, fz = (p.z - g.oz) * g.inv_s;
-    const float before = radius[at];  // an upper bound of the result, or +inf
-    float found = before;
+    float found = radius[at];  // an upper bound of the result, or +inf
     const float most = (float)(rings + 1) / kSearch + g.slack;  // search cells that the cube of +-rings cells spans
-    bool last, full = false;
+    bool last, full;
     float ball = 0.0f;
     do {
       if (found < INFINITY) {
@@ -686,11 +685,12 @@ __global__ void __launch_bounds__(256, K == 4 ? 5 : 4)
       full = __any_sync(0xffffffffu, scanned >= kMaxScan);
     } while (!last && !full);
     if (lane == 0) {
-      radius[at] = full ? fminf(found, before) : found;
       if (full) {  // (the point's place in xyz, marked: n < 2^31)
+        found = fminf(found, radius[at]);
         pending[j] = at | kMark;
         atomicAdd(counts + kMarked, 1u);
       }
+      radius[at] = found;
     }
   }
 }
@@ -700,9 +700,9 @@ __global__ void __launch_bounds__(256, K == 4 ? 5 : 4)
 // first, a cell a lane to look up and the whole warp over each cell's points,
 // until the k-th distance found is within the shells (or a shell is past what
 // is known already: radius holds the best of the first search, or +inf).
-// Sort and search are one cooperative launch, which ends at once where there
-// is no such point: six launches that end at once cost 27 us of a call on a
-// thousand points (131 us), and asking on the host would be a second
+// Sort and search are one cooperative launch, which ends at once (2.7 us) where
+// there is no such point: six launches that end at once cost 27 us of a call on
+// a thousand points (131 us), and asking on the host would be a second
 // synchronisation.
 template <int K>
 __global__ void __launch_bounds__(256, kDenseBlocksPerSm)
@@ -714,6 +714,8 @@ __global__ void __launch_bounds__(256, kDenseBlocksPerSm)
   {
     const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
     const int64_t nt = (m + kScanTile - 1) / kScanTile;
+    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < m; b += (int64_t)gridDim.x * blockDim.x) count[b] = 0u;
+    grid.sync();
     count_points(xyz, n, g, bkt, count);
     grid.sync();
     for (int64_t t = blockIdx.x; t < nt; t += gridDim.x) scan_tile<256>(count, m, t, tiles);
