@@ -251,10 +251,13 @@ constexpr int kPerLane = 4;
 constexpr int kAccumThreads = 128;
 
 // 12 resident blocks per SM (at most 40 registers) where that costs no spills,
-// 10 with five layers, 8 with more.
+// 10 with five layers, 8 with more; with 16 channels 8 (64 registers), 6 with
+// more than five layers.  (Left to the compiler, 16 channels took 107 to 128
+// registers, 4 blocks: frames of 1M points in random order at 640x480 took 88
+// us, now 72; 8M at 1080p 330, 264.)
 template <int C, int kL>
 constexpr int accum_min_blocks() {
-  return C > 8 ? 1 : (kL <= 4 ? 12 : (kL == 5 ? 10 : 8));
+  return C > 8 ? (kL <= 5 ? 8 : 6) : (kL <= 4 ? 12 : (kL == 5 ? 10 : 8));
 }
 
 template <int C, typename TF, int kL>
