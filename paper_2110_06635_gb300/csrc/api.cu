@@ -617,7 +617,7 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
     b.feat_out = params->grad_feat_dtype;
     bool dense = !b.all_projected;
     for (int j = 0; j < nc; ++j) dense = dense && lc.c[j].vis != nullptr;
-    const bool bin = dense && pts->n > 0 && binning_pays(lc, a);
+    const bool bin = dense && pts->n > 0 && binning_pays(lc, a, pts->c);
     if (!bin)
       for (int j = 0; j < nc; ++j) lc.c[j].bin_list = nullptr;
     if (bin &&

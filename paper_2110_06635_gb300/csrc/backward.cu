@@ -983,6 +983,15 @@ __global__ void __launch_bounds__(kReduceThreads) k_bwd_reduce(const float* __re
 cudaError_t launch_bwd_prepass(const LaunchCams& cams, const PointArgs& a, int c, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   const int64_t px = most_pixels(cams, a);
+  // In plain order behind a binning of more than 4800 tiles, whose blocks' 19 KB
+  // of shared memory and more, eight blocks per SM, leave this pass a small L1
+  // if its blocks are placed while they run (4M points, C = 8, early / plain
+  // order: 2800x1600, 4400 tiles, 598 / 619; 3200x1600, 5000 tiles, 680 / 649;
+  // 3000x2250, 6674 tiles, 1160 / 777).
+  int tiles = 0;
+  for (int k = 0; k < a.ncam; ++k)
+    tiles = cams.c[k].bin_list && cams.c[k].tiles > tiles ? cams.c[k].tiles : tiles;
+  const PdlScope pdl(pdl_on() && tiles <= 4800);
   ADOP_DISPATCH_C(c, ADOP_DISPATCH_T((adop_dtype)a.grad_dtype, TG,
                                      e = launch_strided(k_bwd_prepass<kC, TG>, px, a.ncam, kPixelWaves, 0, s, cams,
                                                         a)));
@@ -1024,11 +1033,20 @@ cudaError_t launch_bwd_points(const LaunchCams& cams, const PointArgs& a, const 
 // a CUDA graph, us, binned / in index order, BF16):
 //   20 thousand points, 640x400, surface 60.5 / 48.5, random 65.6 / 46.3
 //   600 thousand, 640x400, surface 88.1 / 80.3, random 116 / 93; 1080p, surface 217 / 221
-//   1.2M, 1080p (590 a tile), surface 269 / 280, random 242 / 200
 //   2.5M, 1080p, surface 317 / 373, random 408 / 400
 //   5M, 640x400, random 247 / 313
-//   1M, 3000x2400 (142 a tile), random 671 / 442
-bool binning_pays(const LaunchCams& cams, const PointArgs& a) {
+// With eight channels and more the pixel records that neighbours share are
+// wider (48 bytes with C = 8, 80 with 16), and binning points that lie in
+// surface order pays from a count on, whatever the tiles (eager step, us):
+//   C = 8, 1080p: 800 thousand 243 / 243, 1M 252 / 265, random 286 / 281
+//   C = 8, 2560x1440: 1.2M 373 / 401, random 419 / 415; 4200x2500: 2M 859 / 962, random 1022 / 1009
+//   C = 16: 300 thousand at 1080p 400 / 400, 400 thousand at 1280x720 271 / 320, 1M at 1080p 537 / 616,
+//   random 614 / 612
+// In random order index order stays ahead below a million points and sixteen
+// channels by up to a quarter; the points' order is not known here, and
+// reconstructed clouds come by surface.
+bool binning_pays(const LaunchCams& cams, const PointArgs& a, int c) {
+  if (c >= 8 && a.n >= (c > 8 ? 300000 : 850000)) return true;
   int most = 0;
   for (int k = 0; k < a.ncam; ++k) most = cams.c[k].tiles > most ? cams.c[k].tiles : most;
   return a.n * a.ncam >= 800000 && a.n >= 500 * (int64_t)most;

@@ -152,7 +152,7 @@ cudaError_t launch_bwd_points(const LaunchCams& cams, const PointArgs& a, const 
 // (The binned point pass then also writes the zero gradients of the points
 // that are in no Lambda when the mode is kGradAssign.)
 // (bits, list and tile offsets; launched where binning_pays.)
-bool binning_pays(const LaunchCams& cams, const PointArgs& a);
+bool binning_pays(const LaunchCams& cams, const PointArgs& a, int c);
 cudaError_t launch_bin(const LaunchCams& cams, const PointArgs& a, const BwdArgs& b, int c, cudaStream_t s);
 // Whether an assigning, binned backward of one camera zeroes all gradients
 // first: with eight points per pyramid pixel (of which one or two can be in
