@@ -461,29 +461,51 @@ def bin_table_bytes(w: int, h: int, sms: int, ncam: int = 1) -> int:
 
 
 def implementation_bytes(kernel: str, n: int, px: int, c: int, s_feat: int, s_out: int,
-                         n_vis: int | None = None, bin_table: int = 0) -> int:
+                         n_vis: int | None = None, bin_table: int = 0, ran=None) -> int:
     """What one launch of this implementation must move (every buffer it
     touches read or written once), including its own records -- the keys it
     reads back, the backward's 16 B pixel records and pixel-major gradient,
     the layer masks and the binning lists.  Not algorithmic bytes: reported
     beside them to show where the design adds traffic (n points, px pyramid
     pixels, c channels, n_vis points in Lambda of at least one layer,
-    bin_table bytes of the binning's block table)."""
+    bin_table bytes of the binning's block table).  ran: the names of the
+    step's kernels -- whether it seeds its sums, bins, and zeroes the gradients
+    ahead decides what each of the others moves; None stands for a seeded,
+    binned step whose zero gradients are the point pass's and whose masks the
+    binning and the point pass read in full."""
     gs = c if c <= 2 else (c + 3) // 4 * 4
     nv = n if n_vis is None else n_vis
-    return {
-        "clear": px * 8,                                        # write key (with a seed pass; else count, sums too)
-        "seed": px * (8 + 4 + 4 * c) + nv * c * s_feat,         # key, the nearest points' tau -> count, sums
+    sums = px * (4 + 4 * c)  # counts and sums
+    seeded = ran is None or "seed" in ran
+    grads = 4 * c + 12
+    out = {
+        "clear": px * 8 + (0 if seeded else sums),              # keys, and what no seed pass will write
+        "seed": px * 8 + sums + nv * c * s_feat,                # key, the nearest points' tau -> count, sums
         "depth": n * (12 + 1) + px * 8 * 2,                     # read xyz -> layer byte; read+write keys
         # xyz, byte -> mask; keys (with a seed pass: the few others' tau and sums are not counted)
         "accumulate": n * (12 + 1 + 4) + px * 8,
-        "normalize": px * (4 + 4 * c + c * s_out),              # read count, sums; write image
-        "bwd_prepass": px * (8 + 4 + 4 * c + 4 * c + 16 + 4 * gs),  # key, count, sums, G -> info, G'
-        "bwd_bin": n * 8 + nv * 4 + 2 * bin_table,                    # masks twice -> list; table written, read
+        "normalize": sums + px * c * s_out,                     # read count, sums; write image
+        "bwd_prepass": px * (8 + 4 * c + 16 + 4 * gs) + sums,   # key, count, sums, G -> info, G'
+        "bwd_bin": n * 8 + nv * 4 + 2 * bin_table,              # masks twice -> list; table written, read
         # list, mask, xyz, tau -> grads of the visible points; pixel records; masks -> zero grads of the rest
-        "bwd_points": nv * (4 + 4 + 12 + c * s_feat + 4 * c + 12) + px * (16 + 4 * gs) + n * 4 + (n - nv) * (4 * c + 12),
+        "bwd_points": nv * (4 + 4 + 12 + c * s_feat + grads) + px * (16 + 4 * gs) + n * 4 + (n - nv) * grads,
+        "bwd_zero": n * grads,
         "bwd_reduce": 0,
-    }.get(kernel, 0)
+    }
+    if ran is not None:
+        bits = (n + 7) // 8
+        # bytes -> masks; xyz and (not seeded) tau of the points in some Lambda, their sums and counts read and written
+        out["accumulate"] = n * (1 + 4) + nv * 12 + px * 8 + (0 if seeded else nv * c * s_feat + 2 * sums)
+        # masks -> bits; bits, the visible points' masks -> list
+        out["bwd_bin"] = n * 4 + 2 * bits + nv * (4 + 4) + 2 * bin_table
+        out["bwd_points"] = nv * (4 + 12 + c * s_feat + grads) + px * (16 + 4 * gs)
+        if "bwd_zero" in ran:
+            out["bwd_points"] += nv * 4                              # the list; the zeros are bwd_zero's
+        elif "bwd_bin" in ran:
+            out["bwd_points"] += nv * 4 + bits + (n - nv) * grads    # the list; bits -> zero grads
+        else:
+            out["bwd_points"] += (n - nv) * (4 + grads)              # the other points' masks -> zero grads
+    return out.get(kernel, 0)
 
 
 def kernel_roofline(ks: dict, n: int, px: int, c: int, s_feat: int, s_out: int, n_vis: int, peak: float,
@@ -497,7 +519,7 @@ def kernel_roofline(ks: dict, n: int, px: int, c: int, s_feat: int, s_out: int, 
     dom = kernel or max(ks, key=lambda k: ks[k][1])
     launches, dom_ms = ks[dom]
     ab = s8d_kernel_bytes(dom, n, px, c, s_feat, s_out)
-    ib = implementation_bytes(dom, n, px, c, s_feat, s_out, n_vis)
+    ib = implementation_bytes(dom, n, px, c, s_feat, s_out, n_vis, ran=ks)
     t = dom_ms / launches * 1e-3
     achieved = ab / t / 1e9
     return {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
@@ -981,7 +1003,7 @@ def bench_large_fwd_bwd(device, sc, steps: int, warmup: int, flush, dtypes=("bf1
                    "roofline": kernel_roofline(ks, wl.n, wl.px, wl.c, wl.s_feat, wl.s_feat, n_vis, peak, peak_kind,
                                                recorded=False),
                    "step_bytes_implementation": sum(implementation_bytes(k, wl.n, wl.px, wl.c, wl.s_feat, wl.s_feat,
-                                                                         n_vis, wl.bin_table) * ks[k][0]
+                                                                         n_vis, wl.bin_table, ran=ks) * ks[k][0]
                                                     for k in ks) // steps,
                    "kernel_ms": {k: round(v[1] / v[0], 4) for k, v in ks.items()}}
         del wl, step
@@ -1209,7 +1231,7 @@ def main():
     roofline = kernel_roofline(ks, wl.n, wl.px, wl.c, wl.s_feat, 2, wl.n_vis, peak, peak_kind)
     kernel_ms = {k: round(v[1] / v[0], 4) for k, v in ks.items()}
     step_bytes = s8d_step_bytes(wl.n, wl.px, wl.c, wl.s_feat, 2)
-    impl_step_bytes = sum(implementation_bytes(k, wl.n, wl.px, wl.c, wl.s_feat, 2, wl.n_vis, wl.bin_table) *
+    impl_step_bytes = sum(implementation_bytes(k, wl.n, wl.px, wl.c, wl.s_feat, 2, wl.n_vis, wl.bin_table, ran=ks) *
                           ks[k][0] for k in ks) // K
     line = {
         "metric": METRIC, "value": round(value, 1), "unit": UNIT, "n_gpus": world, "steps": K,
