@@ -629,7 +629,9 @@ adop_status adop_render_backward(const adop_points* pts, const adop_camera* cams
         (e = timed("bwd_zero", s, [&] { return launch_zero_grads(b, pts->n, pts->c, s); })) != cudaSuccess)
       return cuda_fail(e, "zero gradients launch");
     // the prepass and the point pass that reads its records, a few cameras at a time
-    const int per = cams_per_backward(pts->n, nc);
+    int64_t px = 0;
+    for (int j = 0; j < nc; ++j) px += lc.c[j].off[params->levels];
+    const int per = cams_per_backward(pts->n, nc, px * (16 + 4 * g_stride(pts->c)));
     for (int j0 = 0; j0 < nc; j0 += per) {
       const int m = nc - j0 < per ? nc - j0 : per;
       LaunchCams part;

@@ -96,14 +96,19 @@ struct BwdArgs {
 };
 
 int num_sms();
-// Cameras of one prepass and point pass of a backward over nc cameras: two from
-// 4M points on, where two cameras' launches are long enough to fill the GPU,
-// else all.  The pixel records of two cameras (48 B a pixel at C = 8) are about
-// the L2's size when the point pass reads them, and each camera's blocks are
-// one resident wave.  12 views of 20M points: point passes 1700 us with all in
-// one launch, 1554 by threes, 1354 by twos, 1531 one by one; the prepasses
-// 334, 341, 360, 407; the step 8.46, 8.31, 8.14, 8.35 ms.
-inline int cams_per_backward(int64_t n, int nc) { return n >= ((int64_t)1 << 22) && nc > 2 ? 2 : nc; }
+// Cameras of one prepass and point pass of a backward over nc cameras, whose
+// pixel records (48 B a pixel at C = 8) take `records` bytes in all: two from 4M
+// points on, where two cameras' launches are long enough to fill the GPU, if the
+// records of all are more than the L2 keeps for the point pass, else all.  Each
+// camera's blocks are one resident wave.  12 views of 20M points, 960 MB: point
+// passes 1700 us with all in one launch, 1554 by threes, 1354 by twos, 1531 one
+// by one; the prepasses 334, 341, 360, 407; the step 8.46, 8.31, 8.14, 8.35 ms.
+// Through autograd, all / by twos: 3 views of 5M points, 240 MB, 1168 / 1128 us;
+// 4 of 4.3M, 121 MB, 1014 / 993; 5 of 8M, 51 MB, 1316 / 1351; 16 of 4.3M, 46 MB,
+// 1924 / 2024.
+inline int cams_per_backward(int64_t n, int nc, int64_t records) {
+  return n >= ((int64_t)1 << 22) && nc > 2 && records > ((int64_t)96 << 20) ? 2 : nc;
+}
 // Blocks for a point kernel's items pass: 8 per SM (two waves of its 4
 // resident blocks), shared by the ncam cameras of grid.y.
 int point_blocks(int64_t n, int ncam);

@@ -95,3 +95,36 @@ def test_server_with_seeded_sums(adop, room):
         torch.cuda.synchronize()
         want = np.concatenate([im.cpu().numpy().ravel() for im in fr.images])
         assert_close(o.cpu().numpy(), want, RTOL_FEAT_F32, "image")
+
+
+@pytest.mark.parametrize("keep", [True, False])
+@pytest.mark.parametrize("w,h", [(1100, 900), (320, 200)])
+def test_several_cameras_of_a_large_cloud(adop, w, h, keep):
+    """From 4M points on the backward takes three cameras two at a time where their pixel records (126 MB
+    here, 8 MB) are more than 96 MB: the gradients of one call per camera, summed, and the same pose rows
+    (FP32 sums in another order)."""
+    import torch
+    n = (1 << 22) + 3
+    sc = scenes.tiny_spheres(n, 4, seed=9)
+    cams = [_camera(w, h + 16 * k) for k in range(3)]
+    pts = adop.Points(torch.from_numpy(sc.xyz).cuda(), torch.from_numpy(sc.feat).cuda())
+    params = adop.Params(4, 0.01, 1e-3, None, adop.ADOP_FLAG_GRAD_ASSIGN)
+    G = [[torch.from_numpy(g).cuda() for g in scenes.upstream_grad(c.w, c.h, 4, 4, 30 + k)]
+         for k, c in enumerate(cams)]
+
+    def grads(sub, g):
+        frames = [adop.Frame.alloc(c, 4, 4, torch.float32, keep, "cuda", n if keep else None) for c in sub]
+        ws = adop.alloc_workspace(pts, sub, params)
+        adop.adop_render_forward(pts, sub, params, frames, ws)
+        out = [torch.full((n, 4), float("nan"), device="cuda"), torch.full((n, 3), float("nan"), device="cuda"),
+               torch.zeros((len(sub), 6), device="cuda"), torch.zeros((len(sub), 6), device="cuda")]
+        adop.adop_render_backward(pts, sub, params, frames, g, *out, ws)
+        return [o.cpu().numpy().astype(np.float64) for o in out]
+
+    got = grads(cams, G)
+    one = [grads([c], [g]) for c, g in zip(cams, G)]
+    for j in range(2):
+        assert_close(got[j], sum(o[j] for o in one), 1e-5, "per-point gradients")
+    for j in (2, 3):
+        want = np.concatenate([o[j] for o in one])
+        assert np.all(np.abs(got[j] - want) <= 1e-4 * np.abs(want).max())
