@@ -190,7 +190,8 @@ typedef struct {
  * the 32x32-pixel screen tile of its layer-0 position (row-major over
  * ceil(w/32) tiles per row, position clamped to the image).  The forward
  * writes it; the backward then skips the layers where a point is not in
- * Lambda without looking at any pixel, and visits the points tile by tile.
+ * Lambda without looking at any pixel, and visits the points tile by tile
+ * where there are enough of them for the sort to pay.
  * It is the result of the same FP32 comparisons, so results do not change. */
 typedef struct {
     void* image[ADOP_MAX_LEVELS];
@@ -313,7 +314,8 @@ adop_status adop_pose_apply_tangent(const double* xi, adop_pose* poses, int32_t 
  * one camera each, any resolution -- into caller-owned device buffers.  The
  * only device memory it allocates is one block of mem_budget_bytes at
  * create, from which every admitted request reserves its pixel state
- * (keys, counts, sums: (12 + 4 c) bytes per pyramid pixel).  A scheduler
+ * (keys, counts, sums: (12 + 4 c) bytes per pyramid pixel) and, where that
+ * keeps no request out that could run, a byte per point of its cloud.  A scheduler
  * thread admits queued requests in FIFO order whenever a slot and memory are
  * free, groups the oldest admitted requests (up to max_batch, of any of the
  * resident clouds: each camera of a launch renders its own cloud) into one

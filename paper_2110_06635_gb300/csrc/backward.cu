@@ -668,7 +668,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_bwd_items(const __grid_constant
     // they are: a warp takes 128 points, whose 16 bytes of bits it reads one
     // step ahead, and writes each 32 points that are all zero with 16-byte
     // stores.  (Reading the 4-byte masks again and storing 12 bytes per lane,
-    // the whole pass took 887 us on the 120M-point frame, 807 now.)
+    // the whole pass took 887 us on the 120M-point frame, 807 this way; there
+    // the gradients are zeroed ahead now, zero_first.)
     const int64_t words = (a.n + 31) / 32;
     const int64_t S = (int64_t)gridDim.x * kWarps * 4;
     const bool xyz16 = ((uintptr_t)b.grad_xyz & 15u) == 0u;

@@ -163,8 +163,8 @@ cudaError_t launch_bin(const LaunchCams& cams, const PointArgs& a, const BwdArgs
 // first: with eight points per pyramid pixel (of which one or two can be in
 // some Lambda), from 16M points on, and rows of dL/dtau of at most 16 bytes.
 // 120M points, C = 4: point pass 815 -> 517 + 191 us; 20M in random order, C =
-// 4: 259 -> 88 + 135.  With 32-byte rows the tail already keeps up: 60M points,
-// C = 8: 669 -> 407 + 242, and 16M 170 -> 110 + 72.
+// 4: 259 -> 88 + 135.  With 32-byte rows the tail about keeps up: 60M points,
+// C = 8: 669 -> 407 + 242, but 16M 170 -> 110 + 72.
 inline bool zero_first(int64_t n, int64_t px, int row_bytes) {
   return n >= ((int64_t)1 << 24) && n >= 8 * px && row_bytes <= 16;
 }
