@@ -168,7 +168,9 @@ void Server::admit_locked() {
     state_sum += alloc.round(r.bytes);
     bytes_sum += alloc.round(n);
     const size_t run = std::min((size_t)cfg.max_slots, streams.size() * (size_t)cfg.max_batch);
-    if (bytes_cost_no_request(alloc.capacity(), run, (size_t)active, state_sum, bytes_sum)) r.early = alloc.alloc(n);
+    if (bytes_cost_no_request(alloc.capacity(), alloc.in_use(), run, (size_t)cfg.max_slots, (size_t)active, state_sum,
+                              bytes_sum, alloc.round(n)))
+      r.early = alloc.alloc(n);
   }
 }
 

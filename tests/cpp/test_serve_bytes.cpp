@@ -22,7 +22,10 @@ static std::pair<int, int> admit(const std::vector<std::pair<size_t, size_t>>& r
     ++active;
     state += a.round(r.first);
     bytes += a.round(r.second);
-    if (with && bytes_cost_no_request(a.capacity(), run, (size_t)active, state, bytes) && a.alloc(r.second) != SIZE_MAX)
+    if (with &&
+        bytes_cost_no_request(a.capacity(), a.in_use(), run, (size_t)slots, (size_t)active, state, bytes,
+                              a.round(r.second)) &&
+        a.alloc(r.second) != SIZE_MAX)
       ++got;
   }
   return {active, got};
@@ -45,12 +48,18 @@ int main() {
                           pool, slots, run, w.first, o.first);
               return 1;
             }
-            w.second ? ++granted : ++refused;
+            w.second == w.first ? ++granted : ++refused;  // all with their bytes, or some without
           }
   if (granted < 50 || refused < 50) return std::printf("granted %d, refused %d\n", granted, refused), 1;
   // small views of a large cloud: everything that fitted still does
   const auto small = admit(std::vector<std::pair<size_t, size_t>>(64, {18 * M, 120 * M}), 1200 * M, 32, 64, true);
   if (small.first != 64 || small.second != 0) return std::printf("small: %d, %d\n", small.first, small.second), 1;
+  // a single large view of a large cloud takes them, in a pool that holds seventeen such views
+  const auto one = admit({{486 * M, 50 * M}}, 8590 * M, 32, 64, true);
+  if (one.first != 1 || one.second != 1) return std::printf("one: %d, %d\n", one.first, one.second), 1;
+  // and up to seventeen of these views are admitted as before
+  const std::vector<std::pair<size_t, size_t>> large(64, {486 * M, 50 * M});
+  if (admit(large, 8590 * M, 32, 64, true).first != admit(large, 8590 * M, 32, 64, false).first) return 1;
   // a burst of mixed sizes over a cloud of 8M points has room for all bytes
   std::vector<std::pair<size_t, size_t>> mixed;
   for (int k = 0; k < 16; ++k) mixed.push_back({(size_t[]){18 * M, 54 * M, 121 * M, 486 * M}[k % 4], 8 * M});
